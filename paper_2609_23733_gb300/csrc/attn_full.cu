@@ -68,6 +68,16 @@ constexpr int kCtrlRegs = kChains == 3 ? 56 : 80;
 constexpr int kSoftRegs = kChains == 3 ? 152 : 208;
 static_assert(128 * kCtrlRegs + 128 * kChains * kSoftRegs <= 65536, "register split");
 
+struct Plan {
+  int R, T, S, units;
+  int whole;  // units of the whole-group instance (they come first)
+};
+
+// Units announced by the producer of a split-parts CTA.  Four slots: the MMA warps run at most one
+// tile ahead of the softmax and the producer at most two units ahead of the MMA warps, so slot
+// i is rewritten (unit i + 4) only after every warp has read unit i, however short the units are.
+constexpr int kUnitSlots = 4;
+
 struct FullSmem {
   __nv_bfloat16 q[kChains][kBM * 64];
   __nv_bfloat16 k[kStages][kBN * 64];
@@ -77,6 +87,9 @@ struct FullSmem {
   uint64_t s_full[kChains], s_empty[kChains], p_full[kChains], o_bar[kChains], o_empty[kChains];
   uint64_t drain[kChains];
   uint64_t mufu[kChains][4];  // [chain][SM sub-partition]: that warp finished its exponentials
+  uint64_t unit_full[kUnitSlots];  // split parts: the CTA's next unit (-1: none) is in unit[]
+  int unit[kUnitSlots];
+  Plan plan;
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -89,43 +102,70 @@ struct FullParams {
   float* s_attn;  // [H] MaxAttn saliency (zeroed by the launcher), or NULL
   float* part;    // split-tail partial O, (m, l, xmax) and arrival counters (zeroed)
   float* stats;
-  unsigned int* count;
+  unsigned int* count;  // [kFaCountWords], the last word: units taken (split parts)
   unsigned int* err;
+  int parts_only;       // 1: the split-parts instance runs alone and takes every unit
 };
 
 // The work of one launch: G groups (head, kChains query tiles) over P persistent CTAs.  The
 // first R = floor(G / P) rounds take whole groups; the T = G - R P groups of the last round
-// are split along the keys into S parts each (at most the number of key tiles), T S part
-// units that the P CTAs take round-robin, so the last round lasts ceil(T S / P) parts of a
-// group instead of one whole group on T CTAs.  S minimises ceil(T S / P) (1 / S + c) with c
-// the cost of a part beyond its share of the keys (its Q load, pipeline fill and drain, and
-// the combine), taken as 3 % of a group (0, 1, 3 and 6 % measured within 1 ms of each
-// other on the S = 100 stack, 0 the slowest).  Unit u < R P is group u; unit R P + S t + s is part
-// s of group R P + t.
-struct Plan {
-  int R, T, S, units, whole;  // whole: units that are whole groups (they come first)
-};
-
+// are split along the keys into S parts each (at most the number of key tiles), T S part units,
+// so the last round lasts about ceil(T S / P) parts of a group instead of one whole group on T
+// CTAs.  Unit u < R P is group u; unit R P + S t + s is part s of group R P + t.
+// From kShortTiles key tiles on, S minimises the last round's length in key tiles,
+//   ceil(T S / P) (n_kv / S + kUnitTiles) + kCombineTiles S   (S = 1: no combine).
+// kUnitTiles, the cost of a unit beyond its keys (Q load, pipeline fill and drain, partial store
+// and arrival, about 10 us), and kCombineTiles, what a part adds to the combine (about 1 us), are
+// fitted to a sweep of S at 10,992 tokens; being costs in time they do not shrink with n_kv.
+// Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
+// 10,992 tokens 466 -> 394 us (8 groups left over: 19 parts -> 11), 3 heads 166 -> 122, 1 head at
+// 15,432 tokens 101 -> 92.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
+// 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
+// there: a deep stack of short sequences then gives the same bits as it always did.
 constexpr int kMaxParts = 64;
-constexpr float kPartCost = 0.03f;
+constexpr int kMaxTailUnits = kFaTailUnits * 4 / kChains;  // the scratch is sized for four chains
+constexpr float kUnitTiles = 13.f, kCombineTiles = 1.5f;
+constexpr int kShortTiles = 41;
+constexpr float kPartShare = 0.03f;
 
-__device__ __forceinline__ Plan make_plan(int G, int P, int n_kv) {
+// Called by whole warps: lane l weighs S = l + 1 and l + 33 (a loop over S in every thread took
+// several microseconds of every launch).
+__device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_only) {
+  static_assert(kMaxParts == 64, "two values of S per lane");
   Plan pl;
   pl.R = G / P;
   pl.T = G - pl.R * P;
   pl.S = 1;
   if (pl.T > 0) {
-    float best = 1.f;  // S = 1: the T groups whole, one round
-    for (int S = 2; S <= kMaxParts && S <= n_kv && pl.T * S <= kFaTailUnits; ++S) {
-      const float cost = (float)((pl.T * S + P - 1) / P) * (1.f / (float)S + kPartCost);
-      if (cost < best - 1e-6f) {
+    float best = INFINITY;
+    int bs = 1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int S = lane_id() + 1 + 32 * k;
+      const bool brief = n_kv < kShortTiles;
+      if (S > 1 && (S > n_kv || pl.T * S > (brief ? kFaTailUnits : kMaxTailUnits))) continue;
+      const float rounds = (float)((pl.T * S + P - 1) / P);
+      const float cost = brief ? (S == 1 ? 1.f : rounds * (1.f / (float)S + kPartShare))
+                               : rounds * ((float)n_kv / (float)S + kUnitTiles) +
+                                     (S > 1 ? kCombineTiles * (float)S : 0.f);
+      if (cost < best) {
         best = cost;
-        pl.S = S;
+        bs = S;
       }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {  // smallest cost, then smallest S: the same on every lane
+      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int os = __shfl_xor_sync(0xffffffffu, bs, o);
+      if (ob < best || (ob == best && os < bs)) {
+        best = ob;
+        bs = os;
+      }
+    }
+    pl.S = bs;
   }
   pl.units = pl.S == 1 ? G : pl.R * P + pl.T * pl.S;
-  pl.whole = pl.S == 1 ? G : pl.R * P;
+  pl.whole = parts_only ? 0 : (pl.S == 1 ? G : pl.R * P);
   return pl;
 }
 
@@ -168,11 +208,13 @@ __device__ __forceinline__ Unit unit_of(const Plan& pl, int u, int P, int n_kv) 
 // Split-tail epilogue of one warp (32 rows of chain c, TMEM lanes at t_o): reads the part's
 // unnormalised O rows, releases O_c (o_empty), and publishes them with (m, l, xmax); the last
 // part of this (group, chain, lane quarter) to arrive combines all parts, M = max m_s,
-// O = sum 2^(m_s - M) O_s, l = sum 2^(m_s - M) l_s, and stores Y and the saliency.  Not
-// inlined, and given only values: the attention loop's code and registers stay as they are
-// without it.
-__device__ __noinline__ void split_part(FullParams prm, Plan plan, Unit w, int c, int quarter,
-                                        int lane, int row_in_tile, int row, int h, uint32_t t_o,
+// O = sum 2^(m_s - M) O_s, l = sum 2^(m_s - M) l_s, and stores Y and the saliency.  A part's
+// 32 x 64 block lies lane-minor ([16-byte chunk][lane]), so that every store and load of a warp
+// is 512 contiguous bytes, and the combine works on half a row at a time with the loads of two
+// parts in flight.  Not inlined, and given only values: the attention loop's code and registers
+// stay as they are without it.
+__device__ __noinline__ void split_part(FullParams prm, int S, int part_slot, int tail, int c,
+                                        int quarter, int lane, int row, int h, uint32_t t_o,
                                         uint64_t* o_empty, float m, float lsum, float xmax) {
   float o[64];
   tmem_ld32(t_o, o);
@@ -180,55 +222,90 @@ __device__ __noinline__ void split_part(FullParams prm, Plan plan, Unit w, int c
   tmem_wait_ld();
   tc_fence_before();
   mbar_arrive(o_empty);
-  const size_t prow = (size_t)(w.slot * 4 + c) * kBM + row_in_tile;
-  float4* po = reinterpret_cast<float4*>(prm.part + prow * 64);
+  if (part_slot < 0) {  // a whole group (the parts instance running alone): O / sum -> Y
+    const float inv = 1.f / lsum;
+    if (row < prm.N) {
+      uint4* dst = reinterpret_cast<uint4*>(prm.y + ((size_t)row * prm.H + h) * 64);
 #pragma unroll
-  for (int q = 0; q < 16; ++q) po[q] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-  reinterpret_cast<float4*>(prm.stats)[prow] = make_float4(m, lsum, xmax, 0.f);
+      for (int ch = 0; ch < 8; ++ch) {
+        uint4 v;
+        v.x = pack_bf16x2(o[8 * ch + 0] * inv, o[8 * ch + 1] * inv);
+        v.y = pack_bf16x2(o[8 * ch + 2] * inv, o[8 * ch + 3] * inv);
+        v.z = pack_bf16x2(o[8 * ch + 4] * inv, o[8 * ch + 5] * inv);
+        v.w = pack_bf16x2(o[8 * ch + 6] * inv, o[8 * ch + 7] * inv);
+        dst[ch] = v;
+      }
+    }
+    if (prm.s_attn) {
+      float a = row < prm.N ? fast_exp2(xmax - m) * inv : 0.f;
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, k));
+      if (lane == 0) atomicMax(reinterpret_cast<int*>(prm.s_attn + h), __float_as_int(a));
+    }
+    return;
+  }
+  constexpr size_t kSlot = (size_t)kChains * 4 * 32;  // rows of a slot: [chain][quarter][lane]
+  const size_t blk = (size_t)(c * 4 + quarter) * 32;
+  float4* po = reinterpret_cast<float4*>(prm.part) + (part_slot * kSlot + blk) * 16 + lane;
+#pragma unroll
+  for (int q = 0; q < 16; ++q)
+    po[q * 32] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
+  float4* stats = reinterpret_cast<float4*>(prm.stats) + blk + lane;
+  stats[part_slot * kSlot] = make_float4(m, lsum, xmax, 0.f);
   __threadfence();
   __syncwarp();
   unsigned int last = 0;
   if (lane == 0)
-    last = atomicAdd(prm.count + (w.tail * 4 + c) * 4 + quarter, 1u) == (unsigned)(plan.S - 1);
+    last = atomicAdd(prm.count + (tail * 4 + c) * 4 + quarter, 1u) == (unsigned)(S - 1);
   if (!__shfl_sync(0xffffffffu, last, 0)) return;
   __threadfence();
-  const int slot0 = w.tail * plan.S;
+  const size_t slot0 = (size_t)tail * S;
+  const float4* st = stats + slot0 * kSlot;
   float M = -INFINITY, X = -INFINITY;
-  for (int sp = 0; sp < plan.S; ++sp) {
-    const float4 st4 = __ldcg(reinterpret_cast<const float4*>(prm.stats) +
-                              (size_t)((slot0 + sp) * 4 + c) * kBM + row_in_tile);
+#pragma unroll 8
+  for (int sp = 0; sp < S; ++sp) {
+    const float4 st4 = __ldcg(st + sp * kSlot);
     M = fmaxf(M, st4.x);
     X = fmaxf(X, st4.z);
   }
   float L = 0.f;
-#pragma unroll
-  for (int i = 0; i < 64; ++i) o[i] = 0.f;
-  for (int sp = 0; sp < plan.S; ++sp) {
-    const size_t qrow = (size_t)((slot0 + sp) * 4 + c) * kBM + row_in_tile;
-    const float4 st4 = __ldcg(reinterpret_cast<const float4*>(prm.stats) + qrow);
-    const float wgt = fast_exp2(st4.x - M);
-    L = fmaf(wgt, st4.y, L);
-    const float4* pq = reinterpret_cast<const float4*>(prm.part + qrow * 64);
-#pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const float4 f = __ldcg(pq + q);
-      o[4 * q] = fmaf(wgt, f.x, o[4 * q]);
-      o[4 * q + 1] = fmaf(wgt, f.y, o[4 * q + 1]);
-      o[4 * q + 2] = fmaf(wgt, f.z, o[4 * q + 2]);
-      o[4 * q + 3] = fmaf(wgt, f.w, o[4 * q + 3]);
-    }
+#pragma unroll 8
+  for (int sp = 0; sp < S; ++sp) {
+    const float4 st4 = __ldcg(st + sp * kSlot);
+    L = fmaf(fast_exp2(st4.x - M), st4.y, L);
   }
   const float inv = 1.f / L;
-  if (row < prm.N) {
-    uint4* dst = reinterpret_cast<uint4*>(prm.y + ((size_t)row * prm.H + h) * 64);
+#pragma unroll 1
+  for (int half = 0; half < 2; ++half) {
+    const float4* pq = reinterpret_cast<const float4*>(prm.part) + (slot0 * kSlot + blk) * 16 + lane + half * 256;
+    float acc[32];
 #pragma unroll
-    for (int ch = 0; ch < 8; ++ch) {
-      uint4 v;
-      v.x = pack_bf16x2(o[8 * ch + 0] * inv, o[8 * ch + 1] * inv);
-      v.y = pack_bf16x2(o[8 * ch + 2] * inv, o[8 * ch + 3] * inv);
-      v.z = pack_bf16x2(o[8 * ch + 4] * inv, o[8 * ch + 5] * inv);
-      v.w = pack_bf16x2(o[8 * ch + 6] * inv, o[8 * ch + 7] * inv);
-      dst[ch] = v;
+    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
+#pragma unroll 2
+    for (int sp = 0; sp < S; ++sp) {
+      const float wgt = fast_exp2(__ldcg(&st[sp * kSlot].x) - M);
+      float4 f[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) f[q] = __ldcg(pq + sp * kSlot * 16 + q * 32);
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        acc[4 * q] = fmaf(wgt, f[q].x, acc[4 * q]);
+        acc[4 * q + 1] = fmaf(wgt, f[q].y, acc[4 * q + 1]);
+        acc[4 * q + 2] = fmaf(wgt, f[q].z, acc[4 * q + 2]);
+        acc[4 * q + 3] = fmaf(wgt, f[q].w, acc[4 * q + 3]);
+      }
+    }
+    if (row < prm.N) {
+      uint4* dst = reinterpret_cast<uint4*>(prm.y + ((size_t)row * prm.H + h) * 64) + half * 4;
+#pragma unroll
+      for (int ch = 0; ch < 4; ++ch) {
+        uint4 v;
+        v.x = pack_bf16x2(acc[8 * ch + 0] * inv, acc[8 * ch + 1] * inv);
+        v.y = pack_bf16x2(acc[8 * ch + 2] * inv, acc[8 * ch + 3] * inv);
+        v.z = pack_bf16x2(acc[8 * ch + 4] * inv, acc[8 * ch + 5] * inv);
+        v.w = pack_bf16x2(acc[8 * ch + 6] * inv, acc[8 * ch + 7] * inv);
+        dst[ch] = v;
+      }
     }
   }
   if (prm.s_attn) {
@@ -257,7 +334,19 @@ __global__ void __launch_bounds__(kThreads, 1)
   const int n_groups = (N + kChains * kBM - 1) / (kChains * kBM);  // query-tile groups per head
   const int n_kv = (N + kBN - 1) / kBN;
   const int P = gridDim.x;
-  const Plan plan = make_plan(n_heads * n_groups, P, n_kv);
+  // One warp weighs the splits and hands the plan over in shared memory, from where every warp
+  // reads it as warp-uniform values.
+  if (threadIdx.x < 32) {
+    const Plan p = make_plan(n_heads * n_groups, P, n_kv, prm.parts_only != 0);
+    if (threadIdx.x == 0) sm.plan = p;
+  }
+  __syncthreads();
+  Plan plan;
+  plan.R = __shfl_sync(0xffffffffu, sm.plan.R, 0);
+  plan.T = __shfl_sync(0xffffffffu, sm.plan.T, 0);
+  plan.S = __shfl_sync(0xffffffffu, sm.plan.S, 0);
+  plan.units = __shfl_sync(0xffffffffu, sm.plan.units, 0);
+  plan.whole = __shfl_sync(0xffffffffu, sm.plan.whole, 0);
   // Units of this CTA: [u_begin, u_end) in steps of P.
   const int u_begin = kParts ? plan.whole + (int)blockIdx.x : (int)blockIdx.x;
   const int u_end = kParts ? plan.units : plan.whole;
@@ -292,6 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&sm.drain[c], 1);
       for (int q = 0; q < 4; ++q) mbar_init(&sm.mufu[c][q], 1);
     }
+    for (int i = 0; i < kUnitSlots; ++i) mbar_init(&sm.unit_full[i], 1);
     sm.abort_flag = 0;
     fence_mbarrier_init();
     fence_proxy_async_smem();
@@ -306,6 +396,13 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
+  // The split parts are handed out one at a time (a CTA that starts late, behind a slow whole
+  // group, then takes fewer): unit u_begin first, then from a counter by the producer warp, which
+  // announces them in sm.unit.  Returns the i-th unit of this CTA, -1 after the last.
+  auto announced_unit = [&](uint32_t i, bool& ok) -> int {
+    ok = mbar_wait_warp(&sm.unit_full[i % kUnitSlots], (i / kUnitSlots) & 1, prm.err, abort_flag);
+    return ok ? *reinterpret_cast<volatile int*>(&sm.unit[i % kUnitSlots]) : -1;
+  };
 
   if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kCtrlRegs));
@@ -316,7 +413,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // one elected lane issues the copies.
     uint32_t lc = 0, ic = 0;
     bool ok = true;
-    for (int u = u_begin; u < u_end && ok; u += P, ++ic) {
+    int taken = 0;  // lane 0: the counter's value, read well before it is needed
+    for (int u = u_begin; u < u_end && ok; ++ic) {
+      if constexpr (kParts) {
+        if (elect_one()) {
+          sm.unit[ic % kUnitSlots] = u;
+          mbar_arrive(&sm.unit_full[ic % kUnitSlots]);
+        }
+        __syncwarp();
+        if (lane == 0) taken = (int)atomicAdd(prm.count + kFaCountWords - 1, 1u);
+        __syncwarp();
+      }
       const Unit w = kParts ? unit_of(plan, u, P, n_kv) : whole_unit(u, n_kv);
       const int h = __shfl_sync(0xffffffffu, __ldg(prm.head_ids + first + w.group / n_groups), 0);
       const int qg = w.group % n_groups;
@@ -341,6 +448,15 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         __syncwarp();
       }
+      if (!ok) continue;
+      u = kParts ? plan.whole + P + __shfl_sync(0xffffffffu, taken, 0) : u + P;
+    }
+    if constexpr (kParts) {
+      if (ok && elect_one()) {
+        sm.unit[ic % kUnitSlots] = -1;
+        mbar_arrive(&sm.unit_full[ic % kUnitSlots]);
+      }
+      __syncwarp();
     }
     if (!ok && lane == 0) {
       // Let the copies this warp issued land before the CTA releases its smem.
@@ -372,7 +488,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t lc = 0, ic = 0, g = 0;  // K/V tiles seen, units, S/P/O tiles of this chain
     bool ok = true;
     const int n_kv_all = n_kv;
-    for (int u = u_begin; u < u_end && ok; u += P, ++ic) {
+    for (int u = u_begin; (kParts || u < u_end) && ok; u += P, ++ic) {
+      if constexpr (kParts) {
+        u = announced_unit(ic, ok);
+        if (u < 0) break;
+      }
       const int n_kv = kParts ? unit_of(plan, u, P, n_kv_all).nk : n_kv_all;  // tiles of this unit
       ok = mbar_wait_warp(&sm.q_full, ic & 1, prm.err, abort_flag);
       if (!ok) break;
@@ -381,16 +501,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto issue_s = [&](int j) -> bool {
         const uint32_t l = lc0 + j, gg = g0 + j;
         const int st = l % kStages;
-        if constexpr (kParts) {  // K landed (lanes 0-15 poll) and S_c read (lanes 16-31), at once
-          const bool hi = lane_id() >= 16;
-          if (!__all_sync(0xffffffffu, mbar_wait(hi ? &sm.s_empty[c] : &sm.k_full[st],
-                                                 hi ? ((gg & 1) ^ 1) : ((l / kStages) & 1),
-                                                 prm.err, abort_flag)))
-            return false;
-        } else {
-          if (!mbar_wait_warp(&sm.k_full[st], (l / kStages) & 1, prm.err, abort_flag)) return false;
-          if (!mbar_wait_warp(&sm.s_empty[c], (gg & 1) ^ 1, prm.err, abort_flag)) return false;
-        }
+        if (!mbar_wait_warp(&sm.k_full[st], (l / kStages) & 1, prm.err, abort_flag)) return false;
+        if (!mbar_wait_warp(&sm.s_empty[c], (gg & 1) ^ 1, prm.err, abort_flag)) return false;
         tc_fence_after();
         const uint64_t dk = sdesc_sw128(smem_u32(sm.k[st]));
         if (elect_one()) {
@@ -411,25 +523,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         const uint32_t l = lc0 + j, gg = g0 + j;
         const int st = l % kStages;
-        // P_c written, V landed and, on a unit's first tile, O_c free.  The split parts (short
-        // units) poll the three at once in lane groups (0-10, 11-21, 22-31), so that the round
-        // trips overlap; the whole-group instance waits one after another, which measured
-        // 2.6 % faster there (the same parallel polls in both: stack unchanged, all-full layer
-        // slower).
-        if constexpr (kParts) {
-          const int grp = lane_id() / 11;
-          uint64_t* bar = grp == 0 ? &sm.p_full[c]
-                        : grp == 1 ? &sm.v_full[st]
-                                   : (j == 0 ? &sm.o_empty[c] : &sm.p_full[c]);
-          const uint32_t par = grp == 0 ? (gg & 1)
-                             : grp == 1 ? ((l / kStages) & 1)
-                                        : (j == 0 ? ((ic & 1) ^ 1) : (gg & 1));
-          ok = __all_sync(0xffffffffu, mbar_wait(bar, par, prm.err, abort_flag));
-        } else {
-          ok = mbar_wait_warp(&sm.p_full[c], gg & 1, prm.err, abort_flag) &&
-               mbar_wait_warp(&sm.v_full[st], (l / kStages) & 1, prm.err, abort_flag) &&
-               (j > 0 || mbar_wait_warp(&sm.o_empty[c], (ic & 1) ^ 1, prm.err, abort_flag));
-        }
+        // P_c written, V landed and, on a unit's first tile, O_c free: one wait after another.
+        // (Polling them at once in lane groups measured 2.6 % slower with whole groups and, since
+        // the parts are handed out by a counter, 5 % slower with parts: 1,278 vs 1,187 us for the
+        // parts of two heads at 137,400 tokens.)
+        ok = mbar_wait_warp(&sm.p_full[c], gg & 1, prm.err, abort_flag) &&
+             mbar_wait_warp(&sm.v_full[st], (l / kStages) & 1, prm.err, abort_flag) &&
+             (j > 0 || mbar_wait_warp(&sm.o_empty[c], (ic & 1) ^ 1, prm.err, abort_flag));
         if (!ok) break;
         tc_fence_after();
         const uint64_t dv = sdesc_sw128(smem_u32(sm.v[st]));
@@ -465,9 +565,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t t_p = tmem + lane_off + kColP + c * (kBN / 2);
     const float cs = 1.4426950408889634f * 0.125f;  // log2(e) / sqrt(64)
     const int n_tail = N - (n_kv - 1) * kBN;        // valid keys in the last tile
-    uint32_t g = 0;
+    uint32_t g = 0, ic = 0;
     bool ok = true;
-    for (int u = u_begin; u < u_end && ok; u += P) {
+    for (int u = u_begin; (kParts || u < u_end) && ok; u += P, ++ic) {
+      if constexpr (kParts) {
+        u = announced_unit(ic, ok);
+        if (u < 0) break;
+      }
       const Unit w = kParts ? unit_of(plan, u, P, n_kv) : whole_unit(u, n_kv);
       const int h = __ldg(prm.head_ids + first + w.group / n_groups);
       const int qg = w.group % n_groups;
@@ -578,9 +682,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (!ok) break;
       tc_fence_after();
       const int row = (qg * kChains + c) * kBM + row_in_tile;
-      if (kParts) {  // a part of a split group (the last round's groups)
-        split_part(prm, plan, w, c, quarter, lane, row_in_tile, row, h, t_o, &sm.o_empty[c], m,
-                   lsum, xmax);
+      if (kParts) {  // a part of a split group (the last round's groups), or a whole group
+        split_part(prm, plan.S, w.slot, w.tail, c, quarter, lane, row, h, t_o, &sm.o_empty[c], m, lsum,
+                   xmax);
         __syncwarp();
         continue;
       }
@@ -640,11 +744,19 @@ cudaError_t launch_full_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t s
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(attn_full_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
+  // At most one group per SM even if every head is full: the whole-group instance would find no
+  // round to take unless no group is worth splitting, so the parts instance takes all units and
+  // the other launch is saved.
+  const int groups_max = a.H * ((a.N + kChains * kBM - 1) / (kChains * kBM));
+  const bool parts_only = groups_max <= num_sms;
   FullParams prm{a.N, a.H, a.head_ids, a.offsets, a.y, a.s_attn, a.fa_part, a.fa_stats,
-                 a.fa_count, a.err};
-  attn_full_kernel<false><<<num_sms, kThreads, smem, st>>>(tmap_q, tmap_kv, prm);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+                 a.fa_count, a.err, parts_only ? 1 : 0};
+  if (!parts_only) {
+    attn_full_kernel<false><<<num_sms, kThreads, smem, st>>>(tmap_q, tmap_kv, prm);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    prof_extra_launch();
+  }
   // The split parts of the last round (if the bins give one), on the SMs the whole groups free.
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(num_sms);
@@ -655,9 +767,8 @@ cudaError_t launch_full_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t s
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = parts_only ? 0 : 1;
   e = cudaLaunchKernelEx(&cfg, attn_full_kernel<true>, tmap_q, tmap_kv, prm);
-  prof_extra_launch();
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -36,8 +36,8 @@ struct RouterScratch {
   int32_t* offsets;             // [4]
   unsigned int* cheap_counter;  // work counter of the cheap head modes
   float* lin_state;             // [H][kLinState] linear-attention state (after the router part)
-  float* fa_part;               // [kFaTailUnits][4 chains][128 rows][64] split-tail partial O
-  float* fa_stats;              // [kFaTailUnits][4 chains][128 rows][4] (m, l, xmax, -)
+  float* fa_part;               // split-tail partial O, kFaPartFloats (layout: attn_full.cu)
+  float* fa_stats;              // its (m, l, xmax, -) rows, kFaStatsFloats
   unsigned int* fa_count;       // [kFaTailUnits][4 chains][4 quarters] split arrivals
   float* wo_bias;               // [kMaxHeads * 64] W_O bias with the mean heads folded in
 };
