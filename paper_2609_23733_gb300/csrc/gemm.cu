@@ -2,15 +2,25 @@
 //   out[M][N] = residual + scale (.) act(A[M][K] W[N][K]^T + bias)
 // optionally with a LayerNorm of A's rows folded in (A W^T -> rstd (A W^T - mu c^T), see
 // LinearArgs) and with the output rows' LayerNorm statistics as (mean, M2) per 128 columns.
-// Persistent CTAs (one per SM), 128 x 256 output tiles, 64-wide K blocks through a 4-stage
-// TMA ring (128-byte swizzle), tcgen05.mma (M=128, N=256, K=16, bf16 -> fp32) into one of
-// two TMEM accumulators, so the epilogue of tile i overlaps the main loop of tile i+1.
-// Warp roles: warp 0 TMA, warp 1 TMEM owner + MMA issue, warps 2-9 epilogue: each owns a
-// (32-row TMEM lane quarter, 128-column half) of the tile, one row per thread; per 32-column
-// chunk it loads TMEM (the next chunk's load in flight while this one is processed), applies
-// bias / GELU / LayerScale / residual, packs bf16 into a 64-byte-swizzled 32 x 32 staging
-// block in shared memory and writes it with a TMA tensor store (clipped at the tensor edge).
-// Tiles are visited N-fastest so the CTAs in flight share A rows and all of W in L2.
+// Persistent CTA pairs (clusters of two, cta_group::2), 256 x 256 output tiles: each CTA holds 128
+// rows of A and 128 of W per 64-wide K block in a 5-stage TMA ring (128-byte swizzle, 32 KB a
+// stage), so a K block takes 64 B per clock and SM from L2 where a CTA on its own, with 128 x 256
+// tiles, takes 96 and has a third less look-ahead.  At 137,400 tokens against that design: QKV
+// 529 -> 454 us (1,900 TFLOP/s), FFN-down 683 -> 607, FFN-up + GELU 709 -> 655, W_O with LayerScale
+// and residual 235 -> 183; tensor-bound except W_O, which moves 0.84 GB.  tcgen05.mma (M=256, N=256, K=16, bf16 ->
+// fp32) into one of two TMEM accumulators, so the epilogue of tile i overlaps the main loop of
+// tile i+1.  The tiles of a last round that would use at most half of the pairs are cut into two
+// 128-wide ones each (launch_linear).
+// Warp roles per CTA: warp 0 TMA, warp 1 TMEM owner and (leader CTA) MMA issue, warps 2 ..
+// epilogue (eight or sixteen, launch_linear): each owns a (32-row TMEM lane quarter, half or
+// quarter of the columns) of the tile, one row per thread, the tile's bias and scale in shared
+// memory (from global memory they cost an L2 round trip per chunk); per 32-column chunk it loads TMEM (the next chunk's load in flight while this one
+// is processed), applies bias / GELU / LayerScale / residual, packs bf16 into a 128-byte-swizzled
+// 32 x 64 staging block in shared memory and writes it with a TMA tensor store (clipped at the
+// tensor edge).  The residual comes the same way: its blocks are loaded by TMA into the staging
+// blocks while the tile's MMAs run, and added in place (read row by row from global memory, it
+// took W_O's epilogue longer than the MMAs).
+// Tiles are visited N-fastest so the pairs in flight share A rows and all of W in L2.
 // A second instance (kSkip) leaves chosen 64-column K-blocks out: W_O with the mean heads
 // folded into its bias (wo_mean_fold_kernel) skips their copies and MMAs, and with every block
 // left out it is its epilogue alone.
@@ -23,23 +33,29 @@ namespace vp {
 
 namespace {
 
-constexpr int kBM = 128, kBN = 256, kBK = 64, kStages = 4;
-constexpr int kABytes = kBM * kBK * 2;  // 16 KB
-constexpr int kBBytes = kBN * kBK * 2;  // 32 KB
+constexpr int kBM = 256, kBN = 256, kBK = 64, kStages = 5;  // the pair's tile
+constexpr int kTailN = 128;                                 // width of a cut tile
+constexpr int kABytes = kBM / 2 * kBK * 2;                  // 16 KB: a CTA's half of A
 constexpr uint32_t kTmemCols = 512;
-constexpr int kEpiWarps = 8;
-constexpr int kThreads = 64 + 32 * kEpiWarps;
+constexpr int kBlocks = 16;             // staging blocks, shared out over the epilogue warps
+constexpr int kBlkBytes = 32 * 64 * 2;  // a staging block: 32 rows x 64 columns
 
 struct GemmSmem {
-  __nv_bfloat16 a[kStages][kBM * kBK];
-  __nv_bfloat16 b[kStages][kBN * kBK];
-  __nv_bfloat16 stage[kEpiWarps][2][32 * 32];  // per epilogue warp: two 32 x 32 output blocks
-  uint64_t full[kStages], empty[kStages];
-  uint64_t acc_full[2], acc_empty[2], drain;
+  __nv_bfloat16 a[kStages][kBM / 2 * kBK];
+  __nv_bfloat16 b[kStages][kBN / 2 * kBK];
+  __nv_bfloat16 stage[kBlocks][32 * 64];
+  float vec[2][kBN];        // the tile's bias, and its LayerScale or LN-fold column sums
+  uint64_t full[kStages];   // leader's: both CTAs' copies of a stage have landed
+  uint64_t empty[kStages];
+  uint64_t acc_full[2];
+  uint64_t acc_empty[2];    // leader's: both CTAs' epilogue warps have read the accumulator
+  uint64_t res_full[kBlocks];
+  uint64_t drain;
   uint32_t tmem_base;
   uint32_t skip_mask;  // K-blocks left out (LinearArgs::skip_ids)
   int abort_flag;
 };
+static_assert(sizeof(GemmSmem) <= 232448, "shared memory");
 
 struct GemmParams {
   int M, N, K;
@@ -64,24 +80,43 @@ struct GemmParams {
   const int32_t* tok_index;
   const int32_t* skip_ids;
   const int32_t* skip_off;
+  int full_units, units;  // units 0 .. full_units - 1 are whole tiles, the rest halves of tiles
 };
+
+// Unit u of the launch: the pair's rows from m0, columns [n0, n0 + w).
+struct TileUnit {
+  int m0, n0, w;
+};
+__device__ __forceinline__ TileUnit tile_unit(int u, int full_units, int n_tiles) {
+  const bool cut = u >= full_units;
+  const int t = cut ? full_units + ((u - full_units) >> 1) : u;
+  const int mt = t / n_tiles, nt = t - mt * n_tiles;
+  TileUnit r;
+  r.m0 = mt * kBM;
+  r.n0 = nt * kBN + (cut ? ((u - full_units) & 1) * kTailN : 0);
+  r.w = cut ? kTailN : kBN;
+  return r;
+}
 
 // kSkip: the instance that leaves K-blocks out (GemmParams::skip_ids); the other instance has
 // none of that bookkeeping.
-template <bool kSkip>
-__global__ void __launch_bounds__(kThreads, 1)
+template <bool kSkip, int kEpiWarps>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 const __grid_constant__ CUtensorMap tmap_b,
-                const __grid_constant__ CUtensorMap tmap_out, GemmParams prm) {
-  extern __shared__ unsigned char smem_raw[];
-  GemmSmem& sm = *reinterpret_cast<GemmSmem*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+                const __grid_constant__ CUtensorMap tmap_b_cut,
+                const __grid_constant__ CUtensorMap tmap_out,
+                const __grid_constant__ CUtensorMap tmap_res, GemmParams prm) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  GemmSmem& sm = *reinterpret_cast<GemmSmem*>(smem_raw);
+  constexpr int kParts = kEpiWarps / 4;        // column parts of a tile (epilogue warps per lane quarter)
+  constexpr int kBufs = kBlocks / kEpiWarps;   // staging blocks of a warp = its 64-column groups
   const int M = prm.M, N = prm.N, K = prm.K;
-  const int m_tiles = (M + kBM - 1) / kBM, n_tiles = (N + kBN - 1) / kBN;
-  const int tiles = m_tiles * n_tiles;
+  const int n_tiles = (N + kBN - 1) / kBN;
   const int k_blocks = (K + kBK - 1) / kBK;
-  if ((int)blockIdx.x >= tiles) return;
+  const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
   const int warp = warp_uniform_id(), lane = lane_id();
+  const int rank = __shfl_sync(0xffffffffu, (int)cluster_cta_rank(), 0);
   volatile int* abort_flag = &sm.abort_flag;
 
   if (threadIdx.x == 0) {
@@ -91,8 +126,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&sm.acc_full[b], 1);
-      mbar_init(&sm.acc_empty[b], 32 * kEpiWarps);
+      mbar_init(&sm.acc_empty[b], 2 * kEpiWarps);
     }
+    for (int b = 0; b < kBlocks; ++b) mbar_init(&sm.res_full[b], 1);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
     uint32_t skip = 0;
@@ -106,13 +142,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     tma_prefetch_desc(&tmap_a);
     tma_prefetch_desc(&tmap_b);
     tma_prefetch_desc(&tmap_out);
+    if (prm.residual) tma_prefetch_desc(&tmap_res);
   }
   if (warp == 1) {
-    tmem_alloc(&sm.tmem_base, kTmemCols);
-    tmem_relinquish();
+    tmem_alloc_pair(&sm.tmem_base, kTmemCols);
+    tmem_relinquish_pair();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();  // both CTAs' barriers and TMEM are there
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
   // K-blocks left out, and whether that is all of them (A W^T is then 0).
@@ -120,26 +158,31 @@ __global__ void __launch_bounds__(kThreads, 1)
   const bool acc_zero = kSkip && skip != 0 && __popc(skip & (k_blocks >= 32 ? 0xffffffffu : (1u << k_blocks) - 1u)) == k_blocks;
 
   if (warp == 0) {
-    // TMA producer: converged warp (warp-uniform coordinates), one elected lane issues.
+    // TMA producer of this CTA's halves: converged warp (warp-uniform coordinates), one elected
+    // lane issues.  Both CTAs' copies complete on the leader's barrier, which expects them all.
     uint32_t lc = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-      const int mt = t / n_tiles, nt = t - mt * n_tiles;
+    for (int u = pair; u < prm.units && ok; u += pairs) {
+      const TileUnit t = tile_unit(u, prm.full_units, n_tiles);
+      const bool cut = t.w != kBN;
+      const int row_a = t.m0 + rank * (kBM / 2), row_b = t.n0 + rank * (t.w / 2);
+      const uint32_t bytes = 2 * (kABytes + t.w / 2 * kBK * 2);
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (kSkip && ((skip >> kb) & 1u)) continue;
         const int st = lc % kStages;
         ok = mbar_wait_warp(&sm.empty[st], ((lc / kStages) & 1) ^ 1, prm.err, abort_flag);
         if (!ok) break;
+        const uint32_t full = cluster_addr(&sm.full[st], 0);
         if (elect_one()) {
-          mbar_arrive_expect_tx(&sm.full[st], kABytes + kBBytes);
-          tma_load_2d(sm.a[st], &tmap_a, &sm.full[st], kb * kBK, mt * kBM);
-          tma_load_2d(sm.b[st], &tmap_b, &sm.full[st], kb * kBK, nt * kBN);
+          if (rank == 0) mbar_arrive_expect_tx(&sm.full[st], bytes);
+          tma_load_2d_pair(sm.a[st], &tmap_a, full, kb * kBK, row_a);
+          tma_load_2d_pair(sm.b[st], cut ? &tmap_b_cut : &tmap_b, full, kb * kBK, row_b);
         }
         __syncwarp();
         ++lc;
       }
     }
-    if (!ok && lane == 0) {
+    if (!ok && lane == 0 && rank == 0) {  // both CTAs' copies, as far as they were issued
       for (int s = 0; s < kStages; ++s) {
         if (lc > (uint32_t)s) {
           const uint32_t last = (lc - 1 - s) / kStages * kStages + s;
@@ -148,12 +191,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
     }
   } else if (warp == 1) {
-    // MMA issuer: converged warp; the elected lane (always the lowest, so the same one)
-    // issues the MMAs and the commits that track them.
-    const uint32_t idesc = idesc_bf16(kBM, kBN, 0, 0);
+    // MMA issuer (leader): converged warp; the elected lane (always the lowest, so the same one)
+    // issues the MMAs and the commits that track them, which arrive in both CTAs.
+    const uint32_t id_full = idesc_bf16(kBM, kBN, 0, 0), id_cut = idesc_bf16(kBM, kTailN, 0, 0);
     uint32_t lc = 0, i = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
+    for (int u = pair; rank == 0 && u < prm.units && ok; u += pairs, ++i) {
+      const uint32_t idesc = u >= prm.full_units ? id_cut : id_full;
       const uint32_t ab = i & 1;
       ok = mbar_wait_warp(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1, prm.err, abort_flag);
       if (!ok) break;
@@ -171,30 +215,33 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (elect_one()) {
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk)
-            tc_mma_ss(d, da + 2 * kk, db + 2 * kk, idesc, ((kSkip ? !first : kb > 0) || kk > 0) ? 1u : 0u);
-          tc_commit(&sm.empty[st]);
+            tc_mma_ss_pair(d, da + 2 * kk, db + 2 * kk, idesc, ((kSkip ? !first : kb > 0) || kk > 0) ? 1u : 0u);
+          tc_commit_pair(&sm.empty[st]);
         }
         __syncwarp();
         first = false;
         ++lc;
       }
       if (!ok) break;
-      if (elect_one()) tc_commit(&sm.acc_full[ab]);
+      if (elect_one()) tc_commit_pair(&sm.acc_full[ab]);
       __syncwarp();
     }
     if (!ok) {
       if (elect_one()) {
-        tc_commit(&sm.drain);
+        tc_commit_pair(&sm.drain);
         for (int it = 0; it < 1000000 && !mbar_try_wait(&sm.drain, 0); ++it) {}
       }
       __syncwarp();
     }
   } else {
-    const int e = warp - 2;                 // epilogue warp 0..7
+    const int e = warp - 2;                 // epilogue warp
     const int quarter = warp & 3;           // TMEM lane quarter
-    const int half = e >> 2;                // column half of the tile
+    const int part = e >> 2;                // column part of the tile
     const uint32_t t_lane = tmem + ((uint32_t)(quarter * 32) << 16);
-    unsigned char* stg = reinterpret_cast<unsigned char*>(&sm.stage[e][0][0]);
+    unsigned char* stg = reinterpret_cast<unsigned char*>(&sm.stage[e * kBufs][0]);
+    uint64_t* res_bar = &sm.res_full[e * kBufs];
+    const uint32_t acc_empty0 = cluster_addr(&sm.acc_empty[0], 0);
+    auto epi_sync = []() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
     if (acc_zero) {
       // Every K-block is left out, so no MMA writes the accumulators: zero this thread's
       // columns of both once, and every tile then reads A W^T = 0.
@@ -202,28 +249,57 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int k = 0; k < 32; ++k) z[k] = 0.f;
 #pragma unroll
-      for (int ab = 0; ab < 2; ++ab)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tmem_st32(t_lane + ab * kBN + half * 128 + 32 * q, z);
+      for (int q = 0; q < 16 / kParts; ++q) tmem_st32(t_lane + (part * (16 / kParts) + q) * 32, z);
       tmem_wait_st();
+      // a cut tile's columns are read by other warps of the lane quarter than zeroed them
+      tc_fence_before();
+      epi_sync();
+      tc_fence_after();
     }
     uint32_t i = 0, nst = 0;
-    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
-      const int mt = t / n_tiles, nt = t - mt * n_tiles;
+    for (int u = pair; u < prm.units; u += pairs, ++i) {
+      const TileUnit t = tile_unit(u, prm.full_units, n_tiles);
       const uint32_t ab = i & 1;
-      if (prm.residual) {
-        // Pull this thread's residual row segment (128 columns, 256 bytes) into L2 while the
-        // tile's MMAs still run: read later from HBM, it would hold up the epilogue.
-        const int prow = mt * kBM + quarter * 32 + lane, pcol = nt * kBN + half * 128;
-        if (prow < M && pcol < N) {
-          const __nv_bfloat16* pp = prm.residual + (size_t)prow * N + pcol;
-          asm volatile("prefetch.global.L2 [%0];" ::"l"(pp));
-          if (pcol + 64 < N) asm volatile("prefetch.global.L2 [%0];" ::"l"(pp + 64));
-        }
-      }
-      const int row0 = mt * kBM + quarter * 32;
+      // This warp's columns of the tile: n_grp groups of 64 from pcol0.  A cut tile's two groups
+      // go to the first two parts, or both to the first one where a thread needs a whole
+      // 128-column block (part_out, which runs with two parts).
+      const bool cut = t.w != kBN;
+      const bool both = cut && kParts == 2 && prm.part_out;
+      const int n_grp = !cut ? kBufs : (both ? (part == 0 ? 2 : 0) : (part < 2 ? 1 : 0));
+      const int pcol0 = t.n0 + (both ? 0 : part * (!cut ? kBN / kParts : 64));
+      const int row0 = t.m0 + rank * (kBM / 2) + quarter * 32;
       const int row = row0 + lane;
       const bool row_ok = row < M;
+      // The tile's residual blocks into the staging blocks (once the stores before have read
+      // them) while the tile's MMAs run.
+      if (prm.residual) {
+        if (elect_one()) {
+          tma_store_wait_read<0>();
+          for (int gi = 0; gi < n_grp; ++gi) {
+            if (pcol0 + 64 * gi < N) {
+              const int buf = (nst + gi) % kBufs;
+              mbar_arrive_expect_tx(&res_bar[buf], kBlkBytes);
+              tma_load_2d(stg + buf * kBlkBytes, &tmap_res, &res_bar[buf], pcol0 + 64 * gi, row0);
+            }
+          }
+        }
+        __syncwarp();
+      }
+      // The tile's bias and scale (or LN-fold column sums) into shared memory, a column per
+      // thread: read per chunk from global memory they cost an L2 round trip each.
+      {
+        const int et = (int)threadIdx.x - 64, col = t.n0 + et;
+        const bool in = et < t.w && col < N;
+        const float* second = prm.scale ? prm.scale : prm.ln_c;
+        const float v0 = in && prm.bias ? __ldg(prm.bias + col) : 0.f;
+        const float v1 = in && second ? __ldg(second + col) : 0.f;
+        epi_sync();  // every warp is done with the previous tile's
+        if (et < kBN) {
+          sm.vec[0][et] = v0;
+          sm.vec[1][et] = v1;
+        }
+        epi_sync();
+      }
       // Folded LayerNorm: this row's mean and 1 / sqrt(var + eps) from the (mean, M2) of its
       // 128-column blocks (equal counts: M2 = sum M2_b + 128 sum (mean_b - mean)^2).  The
       // first eight blocks (K = 1,024) are loaded before the accumulator wait.
@@ -239,6 +315,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       const bool ok = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, prm.err, abort_flag);
       if (!ok) break;
       tc_fence_after();
+      // The accumulator goes back to the leader's MMA warp once this warp has read it.
+      auto release_acc = [&]() {
+        tc_fence_before();
+        __syncwarp();
+        if (elect_one()) mbar_arrive_cluster(acc_empty0 + ab * 8);
+      };
+      if (n_grp == 0) {
+        release_acc();
+        continue;
+      }
       if (prm.ln_part && row_ok) {
         float sm_ = 0.f;
 #pragma unroll
@@ -265,18 +351,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         ln_rstd = rsqrtf(m2 / (float)K + prm.ln_eps);
       }
       float cmean[4], cm2[4];  // output statistics per 32-column chunk (part_out)
-      const uint32_t tcol = t_lane + ab * kBN + half * 128;
+      const uint32_t tcol = t_lane + ab * kBN + (pcol0 - t.n0);
       // Bias, or the folded LayerNorm rstd (acc - mu c) + bias', on one 32-column chunk.
       auto bias_fold = [&](float* x, int col0) {
+        const float4* bv = reinterpret_cast<const float4*>(&sm.vec[0][col0 - t.n0]);
         if (prm.ln_part) {  // rstd (acc - mu c) + bias'
+          const float4* cv = reinterpret_cast<const float4*>(&sm.vec[1][col0 - t.n0]);
           const float2 nmu = make_float2(-ln_mu, -ln_mu), rs = make_float2(ln_rstd, ln_rstd);
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            const bool in = col0 + 4 * q + 3 < N;
-            const float4 c4 = in ? __ldg(reinterpret_cast<const float4*>(prm.ln_c + col0) + q)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
-            const float4 b4 = in ? __ldg(reinterpret_cast<const float4*>(prm.bias + col0) + q)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 c4 = cv[q], b4 = bv[q];
             const float2 a0 = ffma2(rs, ffma2(nmu, make_float2(c4.x, c4.y),
                                               make_float2(x[4 * q], x[4 * q + 1])),
                                     make_float2(b4.x, b4.y));
@@ -291,9 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         } else if (prm.bias) {
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
-            const float4 b4 = col0 + 4 * q + 3 < N
-                                  ? __ldg(reinterpret_cast<const float4*>(prm.bias + col0) + q)
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+            const float4 b4 = bv[q];
             const float2 a0 = fadd2(make_float2(x[4 * q], x[4 * q + 1]), make_float2(b4.x, b4.y));
             const float2 a1 = fadd2(make_float2(x[4 * q + 2], x[4 * q + 3]), make_float2(b4.z, b4.w));
             x[4 * q] = a0.x;
@@ -303,33 +385,38 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       };
-      // Stage a 32 x 32 block (row = lane, 64 bytes) and write it with a TMA tensor store.
-      auto store_chunk = [&](const float* x, int col0) {
-        // Stage the 32 x 32 block (row = lane, 64 bytes) in the 64-byte swizzle the
-        // output tensor map uses: 16-byte chunk q of row r sits at chunk q ^ ((r >> 1) & 3).
-        unsigned char* buf = stg + (nst & 1) * 2048;
+      // A 64-column block of the row (row = lane, 128 bytes) lies in the 128-byte swizzle of the
+      // output tensor map: 16-byte chunk q of row r sits at chunk q ^ (r & 7).
+      // Before the first write to it: its last store has read it (with a residual: seen to above).
+      auto block_begin = [&]() -> unsigned char* {
+        unsigned char* buf = stg + (nst % kBufs) * kBlkBytes;
         // The elected lane (lane 0, the lowest) owns this warp's bulk stores and their groups.
-        if (nst >= 2 && elect_one()) tma_store_wait_read<1>();  // this buffer's last store read it
+        if (!prm.residual && nst >= kBufs && elect_one()) tma_store_wait_read<kBufs - 1>();
         __syncwarp();
+        return buf + lane * 128;
+      };
+      // 32 columns (chunks 4 hc .. 4 hc + 3 of the row), packed to bf16.
+      auto block_put = [&](unsigned char* brow, const float* x, int hc) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          uint4 u;
-          u.x = pack_bf16x2(x[8 * q + 0], x[8 * q + 1]);
-          u.y = pack_bf16x2(x[8 * q + 2], x[8 * q + 3]);
-          u.z = pack_bf16x2(x[8 * q + 4], x[8 * q + 5]);
-          u.w = pack_bf16x2(x[8 * q + 6], x[8 * q + 7]);
-          *reinterpret_cast<uint4*>(buf + lane * 64 + ((q ^ ((lane >> 1) & 3)) << 4)) = u;
+          uint4 v;
+          v.x = pack_bf16x2(x[8 * q + 0], x[8 * q + 1]);
+          v.y = pack_bf16x2(x[8 * q + 2], x[8 * q + 3]);
+          v.z = pack_bf16x2(x[8 * q + 4], x[8 * q + 5]);
+          v.w = pack_bf16x2(x[8 * q + 6], x[8 * q + 7]);
+          *reinterpret_cast<uint4*>(brow + (((4 * hc + q) ^ (lane & 7)) << 4)) = v;
         }
+      };
+      auto block_store = [&](int col0) {
         fence_proxy_async_smem();
         __syncwarp();
         if (elect_one()) {
-          tma_store_2d(&tmap_out, buf, col0, row0);
+          tma_store_2d(&tmap_out, stg + (nst % kBufs) * kBlkBytes, col0, row0);
           tma_store_commit();
         }
         ++nst;
       };
-      const int pcol0 = nt * kBN + half * 128;  // this thread's 128 columns: two heads
-      if (prm.qk_cols > 0 && pcol0 < prm.qk_cols) {
+      if (kParts == 2 && prm.qk_cols > 0 && pcol0 < prm.qk_cols) {
         // Q or K columns of a QKV projection with qk-norm and / or 2-D RoPE: whole heads
         // (64 columns, two chunks) at a time.
         const bool is_q = pcol0 < (prm.qk_cols >> 1);
@@ -345,15 +432,12 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
 #pragma unroll 1
-        for (int hh = 0; hh < 2; ++hh) {
+        for (int hh = 0; hh < n_grp; ++hh) {
           float x[64];
           tmem_ld32(tcol + 64 * hh, x);
           tmem_ld32(tcol + 64 * hh + 32, x + 32);
           tmem_wait_ld();
-          if (hh == 1) {
-            tc_fence_before();
-            mbar_arrive(&sm.acc_empty[ab]);
-          }
+          if (hh == n_grp - 1) release_acc();
           const int col0 = pcol0 + 64 * hh;
           bias_fold(x, col0);
           bias_fold(x + 32, col0 + 32);
@@ -402,20 +486,33 @@ __global__ void __launch_bounds__(kThreads, 1)
               }
             }
           }
-          if (col0 < N) store_chunk(x, col0);
-          if (col0 + 32 < N) store_chunk(x + 32, col0 + 32);
+          if (col0 < N) {
+            unsigned char* brow = block_begin();
+            block_put(brow, x, 0);
+            block_put(brow, x + 32, 1);
+            block_store(col0);
+          }
         }
         continue;
       }
       float v[2][32];
       tmem_ld32(tcol, v[0]);
       tmem_wait_ld();
+      unsigned char* brow = nullptr;
 #pragma unroll
-      for (int cc = 0; cc < 4; ++cc) {
-        if (cc + 1 < 4) tmem_ld32(tcol + 32 * (cc + 1), v[(cc + 1) & 1]);  // in flight meanwhile
+      for (int cc = 0; cc < 2 * kBufs; ++cc) {
+        if (cc >= 2 * n_grp) break;
+        if (cc + 1 < 2 * n_grp) tmem_ld32(tcol + 32 * (cc + 1), v[(cc + 1) & 1]);  // in flight meanwhile
         float* x = v[cc & 1];
-        const int col0 = nt * kBN + half * 128 + cc * 32;
-        if (col0 < N) {
+        const int col0 = pcol0 + cc * 32;
+        const bool live = pcol0 + 64 * (cc >> 1) < N;  // the 64-column block has columns to store
+        if (live) {
+          if ((cc & 1) == 0) {
+            brow = block_begin();
+            if (prm.residual &&
+                !mbar_wait_warp(&res_bar[nst % kBufs], (nst / kBufs) & 1, prm.err, abort_flag))
+              break;
+          }
           // Bias, GELU, LayerScale and residual on column pairs (packed f32x2 arithmetic).
           bias_fold(x, col0);
           if (prm.act == VP_ACT_GELU) {
@@ -429,9 +526,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           if (prm.scale) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-              const float4 s4 = col0 + 4 * q + 3 < N
-                                    ? __ldg(reinterpret_cast<const float4*>(prm.scale + col0) + q)
-                                    : make_float4(0.f, 0.f, 0.f, 0.f);
+              const float4 s4 = reinterpret_cast<const float4*>(&sm.vec[1][col0 - t.n0])[q];
               const float2 a0 = fmul2(make_float2(x[4 * q], x[4 * q + 1]), make_float2(s4.x, s4.y));
               const float2 a1 = fmul2(make_float2(x[4 * q + 2], x[4 * q + 3]), make_float2(s4.z, s4.w));
               x[4 * q] = a0.x;
@@ -440,24 +535,21 @@ __global__ void __launch_bounds__(kThreads, 1)
               x[4 * q + 3] = a1.y;
             }
           }
-          if (prm.residual && row_ok) {
-            const __nv_bfloat16* rp = prm.residual + (size_t)row * N + col0;
+          if (prm.residual) {  // rows and columns past the edge were filled with zeros
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-              if (col0 + 8 * q + 7 < N) {
-                const uint4 u = *reinterpret_cast<const uint4*>(rp + 8 * q);
-                const uint32_t uw[4] = {u.x, u.y, u.z, u.w};
+              const uint4 ru = *reinterpret_cast<const uint4*>(brow + (((4 * (cc & 1) + q) ^ (lane & 7)) << 4));
+              const uint32_t uw[4] = {ru.x, ru.y, ru.z, ru.w};
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                  const float2 a = fadd2(make_float2(x[8 * q + 2 * k], x[8 * q + 2 * k + 1]),
-                                         make_float2(bf16_lo(uw[k]), bf16_hi(uw[k])));
-                  x[8 * q + 2 * k] = a.x;
-                  x[8 * q + 2 * k + 1] = a.y;
-                }
+              for (int k = 0; k < 4; ++k) {
+                const float2 a = fadd2(make_float2(x[8 * q + 2 * k], x[8 * q + 2 * k + 1]),
+                                       make_float2(bf16_lo(uw[k]), bf16_hi(uw[k])));
+                x[8 * q + 2 * k] = a.x;
+                x[8 * q + 2 * k + 1] = a.y;
               }
             }
           }
-          if (prm.part_out) {  // chunk mean and M2 (two passes over registers)
+          if (kParts == 2 && prm.part_out) {  // chunk mean and M2 (two passes over registers)
             float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < 16; ++k) s2 = fadd2(s2, make_float2(x[2 * k], x[2 * k + 1]));
@@ -471,16 +563,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             cmean[cc] = cm;
             cm2[cc] = q2.x + q2.y;
           }
-          store_chunk(x, col0);
+          block_put(brow, x, cc & 1);
+          if (cc & 1) block_store(pcol0 + 64 * (cc >> 1));
         }
         tmem_wait_ld();
-        if (cc == 3) {
-          tc_fence_before();
-          mbar_arrive(&sm.acc_empty[ab]);
-        }
+        if (cc + 2 == 2 * n_grp) release_acc();  // the last chunk is in registers
       }
-      const int pcol = nt * kBN + half * 128;  // this thread's 128-column block
-      if (prm.part_out && row_ok && pcol < N) {
+      const int pcol = pcol0;  // this thread's 128-column block
+      if (kParts == 2 && prm.part_out && row_ok && pcol < N) {
         const float mb = 0.25f * (cmean[0] + cmean[1] + cmean[2] + cmean[3]);
         float m2 = cm2[0] + cm2[1] + cm2[2] + cm2[3];
 #pragma unroll
@@ -488,15 +578,16 @@ __global__ void __launch_bounds__(kThreads, 1)
         prm.part_out[(size_t)row * (N >> 7) + (pcol >> 7)] = make_float2(mb, m2);
       }
     }
-    if (elect_one()) tma_store_wait_all();
+    if (elect_one()) tma_store_wait_read<0>();  // the staging blocks outlive the reads
     __syncwarp();
   }
 
   tc_fence_before();
   __syncthreads();
+  cluster_sync_all();  // neither CTA leaves while the other uses its shared memory or TMEM
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc_pair(tmem, kTmemCols);
   }
 }
 
@@ -554,19 +645,20 @@ cudaError_t launch_wo_mean_fold(int D, int H, const __nv_bfloat16* w_o, const fl
 }
 
 cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
-  CUtensorMap ta, tb, to;
-  cudaError_t e = make_tmap_bf16_2d(&ta, a.A, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.K, kBK, kBM);
+  CUtensorMap ta, tb, tb_cut, to, tr;
+  cudaError_t e = make_tmap_bf16_2d(&ta, a.A, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.K, kBK, kBM / 2);
   if (e != cudaSuccess) return e;
-  e = make_tmap_bf16_2d(&tb, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kBN);
+  e = make_tmap_bf16_2d(&tb, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kBN / 2);
   if (e != cudaSuccess) return e;
-  e = make_tmap_bf16_2d(&to, a.out, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N, 32, 32, 64);
+  e = make_tmap_bf16_2d(&tb_cut, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kTailN / 2);
   if (e != cudaSuccess) return e;
-  const int smem = (int)sizeof(GemmSmem) + 1024;
-  const bool skip = a.skip_ids != nullptr;
-  e = cudaFuncSetAttribute(skip ? gemm_kernel<true> : gemm_kernel<false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  e = make_tmap_bf16_2d(&to, a.out, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N, 64, 32);
   if (e != cudaSuccess) return e;
-  const int tiles = ((a.M + kBM - 1) / kBM) * ((a.N + kBN - 1) / kBN);
+  tr = to;
+  if (a.residual && a.residual != a.out) {
+    e = make_tmap_bf16_2d(&tr, a.residual, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N, 64, 32);
+    if (e != cudaSuccess) return e;
+  }
   if ((a.ln_part && (a.K % 256 != 0 || !a.ln_c || !a.bias)) ||
       (a.part_out && a.N % 128 != 0))
     return cudaErrorInvalidValue;
@@ -577,17 +669,39 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
              a.residual || a.part_out || (!a.qn_g != !a.qn_b) || (!a.kn_g != !a.kn_b) ||
              (a.rope_cs && (a.tok_per_view < 1 || a.grid_w < 1 || a.patch_start < 0))))
     return cudaErrorInvalidValue;
+  // Whole rounds of 256 x 256 tiles over the pairs; a last round that at most half of the pairs
+  // would work on is cut into tiles of half the width (10,992 x 1,024 from K = 4,096: 172 tiles
+  // on 76 pairs; 1,044 rows: 20 tiles become 40, K = 4,096 28.0 us with 128 x 256 tiles of single
+  // CTAs, 16.5 here).
+  const int pairs_max = max(1, num_sms / 2);
+  const int tiles = ((a.M + kBM - 1) / kBM) * ((a.N + kBN - 1) / kBN);
+  const int left = tiles % pairs_max;
+  const int full_units = 2 * left <= pairs_max ? tiles - left : tiles;
+  const int units = full_units + 2 * (tiles - full_units);
   GemmParams prm{a.M,     a.N,   a.K,   a.bias,      a.act,  a.scale,   a.residual,
                  a.out,   a.err, a.ln_part, a.ln_c, a.ln_eps, a.part_out,
                  qk ? a.qk_cols : 0, a.qn_g, a.qn_b, a.kn_g, a.kn_b, a.qk_eps, a.rope_cs,
-                 a.tok_per_view, a.patch_start, a.grid_w, a.tok_index, a.skip_ids, a.skip_off};
-  prof_before(VP_KERNEL_GEMM, st);
-  if (skip)
-    gemm_kernel<true><<<min(num_sms, tiles), kThreads, smem, st>>>(ta, tb, to, prm);
-  else
-    gemm_kernel<false><<<min(num_sms, tiles), kThreads, smem, st>>>(ta, tb, to, prm);
-  prof_after(st);
-  return cudaGetLastError();
+                 a.tok_per_view, a.patch_start, a.grid_w, a.tok_index, a.skip_ids, a.skip_off,
+                 full_units, units};
+  const int grid = 2 * min(pairs_max, units);
+  const int smem = (int)sizeof(GemmSmem);
+  auto launch = [&](auto kernel, int epi_warps) -> cudaError_t {
+    cudaError_t le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (le != cudaSuccess) return le;
+    prof_before(VP_KERNEL_GEMM, st);
+    kernel<<<grid, 64 + 32 * epi_warps, smem, st>>>(ta, tb, tb_cut, to, tr, prm);
+    prof_after(st);
+    return cudaGetLastError();
+  };
+  // Sixteen epilogue warps (64 columns of a row per thread, one staging block each) where the
+  // epilogue is what a tile waits for: GELU (137,400 x 4,096 from K = 1,024: 668 us with eight
+  // warps, 655 with sixteen), and a single round, whose epilogue no next tile covers (1,044 x
+  // 1,024 with residual 15.4 -> 12.2 us).  Eight elsewhere (128 columns, two blocks, so that the
+  // next tile's residual loads start earlier: 137,400 x 1,024 with residual 183 us against 189,
+  // x 3,072 454 against 462); qk-norm and part_out need a thread to hold whole heads or blocks.
+  const bool sixteen = !a.part_out && !qk && (a.act == VP_ACT_GELU || units <= pairs_max);
+  if (a.skip_ids) return sixteen ? launch(gemm_kernel<true, 16>, 16) : launch(gemm_kernel<true, 8>, 8);
+  return sixteen ? launch(gemm_kernel<false, 16>, 16) : launch(gemm_kernel<false, 8>, 8);
 }
 
 }  // namespace vp
