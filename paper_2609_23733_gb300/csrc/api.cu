@@ -308,12 +308,15 @@ SurrogateArgs make_surrogate_args(const vp_surrogate_weights* sw) {
 }
 
 // Runs the three mode kernels for bins already in device memory.
+// in_layer: the router just before cleared the counters (and s_attn).
 // skip_mean_y: the mean heads' rows of Y are left unwritten (their part of W_O is folded into
-// its bias, launch_wo_mean_fold).
+// its bias: here if wo_bias is given, else by launch_wo_mean_fold).
 vp_status run_heads(const vp_dims* dm, const __nv_bfloat16* qkv, const int32_t* head_ids,
                     const int32_t* offsets, const float* ctx, const float* mean_v,
                     const vp_surrogate_weights* sw, __nv_bfloat16* y, float* s_attn,
-                    const RouterScratch& sc, cudaStream_t st, bool skip_mean_y = false) {
+                    const RouterScratch& sc, cudaStream_t st, bool in_layer = false,
+                    bool skip_mean_y = false, const __nv_bfloat16* w_o = nullptr,
+                    const float* b_o = nullptr, float* wo_bias = nullptr) {
   HeadAttnArgs ha{};
   ha.N = dm->N;
   ha.H = dm->H;
@@ -332,7 +335,11 @@ vp_status run_heads(const vp_dims* dm, const __nv_bfloat16* qkv, const int32_t* 
   ha.y = y;
   ha.s_attn = s_attn;
   ha.err = sc.err;
-  ha.cheap_counter = sc.cheap_counter;
+  ha.cheap_counter = sc.fa_count + kCheapCounter;
+  ha.counters_zeroed = in_layer ? 1 : 0;
+  ha.w_o = w_o;
+  ha.b_o = b_o;
+  ha.wo_bias = wo_bias;
   ha.skip_mean_y = skip_mean_y ? 1 : 0;
   return from_cuda(launch_heads(ha, device_sm_count(), st));
 }
@@ -380,14 +387,23 @@ vp_status run_layer(const vp_dims* dm, const __nv_bfloat16* xin, const vp_bf16* 
   RouterArgs ra = make_router_args(dm, reinterpret_cast<const vp_bf16*>(qkv), rw, force_modes);
   ra.s_out = s_out;
   ra.modes_out = modes_out;
+  ra.zero = sc.fa_count;
+  ra.zero_words = (int)kFaCountWords;
+  ra.s_attn_zero = s_attn_out;
   VP_TRY(from_cuda(launch_router(ra, sc, sms, st)));
-  prof_before(VP_KERNEL_GEMM, st);  // W_O's bias, counted with the projections
-  const cudaError_t ef = launch_wo_mean_fold(D, dm->H, reinterpret_cast<const __nv_bfloat16*>(w_o),
-                                             b_o, sc.mean_v, sc.head_ids, sc.offsets, sc.wo_bias, st);
-  prof_after(st);
-  VP_TRY(from_cuda(ef));
+  const __nv_bfloat16* wo = reinterpret_cast<const __nv_bfloat16*>(w_o);
+  // W_O's bias with the mean heads: by the cheap-heads kernel, or on its own where a variant
+  // does not run that kernel.
+  const bool fold_alone = dm->variant & (VP_VARIANT_NO_RESIDUAL | VP_VARIANT_LINEAR_ATTENTION);
+  if (fold_alone) {
+    prof_before(VP_KERNEL_GEMM, st);  // counted with the projections
+    const cudaError_t ef = launch_wo_mean_fold(D, dm->H, wo, b_o, sc.mean_v, sc.head_ids, sc.offsets,
+                                               sc.wo_bias, st);
+    prof_after(st);
+    VP_TRY(from_cuda(ef));
+  }
   VP_TRY(run_heads(dm, qkv, sc.head_ids, sc.offsets, sc.ctx, sc.mean_v, sw, y, s_attn_out, sc,
-                   st, !keep_mean_y));
+                   st, true, !keep_mean_y, wo, b_o, fold_alone ? nullptr : sc.wo_bias));
   LinearArgs lo{};
   lo.M = N;
   lo.N = D;
@@ -731,7 +747,7 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
     if (!w.merge)
       VP_TRY(from_cuda(launch_ln_fold_weights(3 * D, D,
                                               reinterpret_cast<const __nv_bfloat16*>(w.w_qkv),
-                                              w.ln1_g, w.ln1_b, w.b_qkv, wq, cq, bq, st)));
+                                              w.ln1_g, w.ln1_b, w.b_qkv, wq, cq, bq, true, st)));
     if (w.qk && w.qk->rope &&
         !(rope_built && rope_built->rope_base == w.qk->rope_base &&
           rope_built->tokens_per_view == w.qk->tokens_per_view &&

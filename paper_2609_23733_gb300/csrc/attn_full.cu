@@ -26,8 +26,8 @@
 // TMEM: S_c at [c kBN, +kBN), O_c at [kChains kBN + 64 c, +64), P_c after the O columns.
 // Keys past N are zero-filled by TMA and masked to -inf; query rows past N are not stored.
 // Optionally the epilogue also yields the head's MaxAttn saliency max_ij A_ij (§3).
-// Every CTA signals its dependents at once (griddepcontrol.launch_dependents), so the
-// cheap-heads kernel queued behind this one (heads_cheap.cu) can take the SMs that the last
+// Every CTA signals its dependents as soon as everything before this kernel has completed, so
+// the cheap-heads kernel queued behind this one (heads_cheap.cu) can take the SMs that the last
 // full-attention round leaves idle.
 // Every mbarrier wait is bounded (mbar_wait); on timeout the CTA records the error, stops
 // issuing work, waits (bounded) for its own outstanding copies and MMAs, frees TMEM, exits.
@@ -102,7 +102,7 @@ struct FullParams {
   float* s_attn;  // [H] MaxAttn saliency (zeroed by the launcher), or NULL
   float* part;    // split-tail partial O, (m, l, xmax) and arrival counters (zeroed)
   float* stats;
-  unsigned int* count;  // [kFaCountWords], the last word: units taken (split parts)
+  unsigned int* count;  // [kFaCountWords] arrivals per (group, chain, quarter); units taken
   unsigned int* err;
   int parts_only;       // 1: the split-parts instance runs alone and takes every unit
 };
@@ -328,8 +328,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   FullSmem& sm = *reinterpret_cast<FullSmem*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
 
-  const int first = __ldg(prm.offsets + 2);
-  const int n_heads = __ldg(prm.offsets + 3) - first;
+  // The first attention kernel of a layer waits for the kernel before it (the bins); the split
+  // parts behind the whole groups start only once those have waited, and run beside them.
+  if (!kParts || prm.parts_only) pdl_wait();
+  const int first = prm.offsets[2];
+  const int n_heads = prm.offsets[3] - first;
   const int N = prm.N, H = prm.H;
   const int n_groups = (N + kChains * kBM - 1) / (kChains * kBM);  // query-tile groups per head
   const int n_kv = (N + kBN - 1) / kBN;
@@ -354,15 +357,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     // The parts grid completes only after the whole-group grid (its prerequisite): work
     // queued behind it then sees every row of Y.
     if (kParts && blockIdx.x == 0) {
-      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-      asm volatile("griddepcontrol.wait;" ::: "memory");
+      pdl_launch();
+      pdl_wait();
     }
     return;
   }
 
   const int warp = warp_uniform_id(), lane = lane_id();
   volatile int* abort_flag = &sm.abort_flag;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  pdl_launch();
 
   if (threadIdx.x == 0) {
     mbar_init(&sm.q_full, 1);
@@ -421,11 +424,11 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive(&sm.unit_full[ic % kUnitSlots]);
         }
         __syncwarp();
-        if (lane == 0) taken = (int)atomicAdd(prm.count + kFaCountWords - 1, 1u);
+        if (lane == 0) taken = (int)atomicAdd(prm.count + kFaUnitCounter, 1u);
         __syncwarp();
       }
       const Unit w = kParts ? unit_of(plan, u, P, n_kv) : whole_unit(u, n_kv);
-      const int h = __shfl_sync(0xffffffffu, __ldg(prm.head_ids + first + w.group / n_groups), 0);
+      const int h = __shfl_sync(0xffffffffu, prm.head_ids[first + w.group / n_groups], 0);
       const int qg = w.group % n_groups;
       ok = mbar_wait_warp(&sm.q_empty, (ic & 1) ^ 1, prm.err, abort_flag);
       if (!ok) break;
@@ -573,7 +576,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (u < 0) break;
       }
       const Unit w = kParts ? unit_of(plan, u, P, n_kv) : whole_unit(u, n_kv);
-      const int h = __ldg(prm.head_ids + first + w.group / n_groups);
+      const int h = prm.head_ids[first + w.group / n_groups];
       const int qg = w.group % n_groups;
       // m: the (lazily updated) reference the exponentials are taken against; xmax: the
       // true running maximum of the row's scaled scores, for the MaxAttn saliency.
@@ -726,7 +729,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
   }
-  if (kParts && blockIdx.x == 0 && threadIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (kParts && blockIdx.x == 0 && threadIdx.x == 0) pdl_wait();
 }
 
 }  // namespace
@@ -752,25 +755,12 @@ cudaError_t launch_full_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t s
   FullParams prm{a.N, a.H, a.head_ids, a.offsets, a.y, a.s_attn, a.fa_part, a.fa_stats,
                  a.fa_count, a.err, parts_only ? 1 : 0};
   if (!parts_only) {
-    attn_full_kernel<false><<<num_sms, kThreads, smem, st>>>(tmap_q, tmap_kv, prm);
-    e = cudaGetLastError();
+    e = launch_pdl(attn_full_kernel<false>, dim3(num_sms), kThreads, smem, st, tmap_q, tmap_kv, prm);
     if (e != cudaSuccess) return e;
     prof_extra_launch();
   }
   // The split parts of the last round (if the bins give one), on the SMs the whole groups free.
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(num_sms);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = parts_only ? 0 : 1;
-  e = cudaLaunchKernelEx(&cfg, attn_full_kernel<true>, tmap_q, tmap_kv, prm);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  return launch_pdl(attn_full_kernel<true>, dim3(num_sms), kThreads, smem, st, tmap_q, tmap_kv, prm);
 }
 
 }  // namespace vp

@@ -149,6 +149,19 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// ---------------------------------------------------------------- programmatic dependent launch
+// Kernels of a call are launched with launch_pdl (internal.h): a kernel may start while the one
+// before it still runs, sets up what touches no global memory, and waits.  pdl_wait returns
+// once the kernel before has completed and its writes are visible; as every kernel waits (all
+// of it, or at least one thread before the grid ends), everything earlier in the stream has
+// completed too.  What an earlier kernel wrote is read with plain loads, never __ldg: the compiler
+// may move a read-only load above the wait.  pdl_launch, after the wait, lets the next kernel start: what that one does
+// before its own wait can rely on every kernel before this one.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- tcgen05
 __device__ __forceinline__ void tmem_alloc(uint32_t* smem_result, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -418,6 +431,29 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 
 __device__ __forceinline__ float bf16_lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
+
+// Column n of W_O's bias with the mean heads folded in (internal.h, launch_wo_mean_fold), by one
+// warp: lane l takes channels 2 l, 2 l + 1 of the mean heads head_ids[m0 .. m1).
+__device__ __forceinline__ void wo_mean_fold_column(int n, int H, const __nv_bfloat16* w_o,
+                                                    const float* b_o, const float* mean_v,
+                                                    const int32_t* head_ids, int m0, int m1,
+                                                    float* bias_out) {
+  const int lane = threadIdx.x & 31;
+  const __nv_bfloat16* wrow = w_o + (size_t)n * H * 64 + 2 * lane;
+  float acc = 0.f;
+#pragma unroll 4
+  for (int i = m0; i < m1; ++i) {
+    const int h = head_ids[i];
+    const uint32_t w2 = *reinterpret_cast<const unsigned int*>(wrow + h * 64);
+    // the mean head's row of Y as stored: bf16(mean_v), round to nearest even
+    const float2 mv = reinterpret_cast<const float2*>(mean_v + h * 64)[lane];
+    const uint32_t mu = pack_bf16x2(mv.x, mv.y);
+    acc = fmaf(bf16_lo(mu), bf16_lo(w2), fmaf(bf16_hi(mu), bf16_hi(w2), acc));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) bias_out[n] = (b_o ? b_o[n] : 0.f) + acc;
+}
 
 __device__ __forceinline__ float fast_exp2(float x) {
   float y;

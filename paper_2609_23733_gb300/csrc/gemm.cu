@@ -131,12 +131,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     for (int b = 0; b < kBlocks; ++b) mbar_init(&sm.res_full[b], 1);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
-    uint32_t skip = 0;
-    if (kSkip) {
-      const int s0 = __ldg(prm.skip_off), s1 = __ldg(prm.skip_off + 1);
-      for (int i = s0; i < s1; ++i) skip |= 1u << (__ldg(prm.skip_ids + i) & 31);
-    }
-    sm.skip_mask = skip;
     fence_mbarrier_init();
     fence_proxy_async_smem();
     tma_prefetch_desc(&tmap_a);
@@ -147,6 +141,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
   if (warp == 1) {
     tmem_alloc_pair(&sm.tmem_base, kTmemCols);
     tmem_relinquish_pair();
+  }
+  pdl_wait();
+  pdl_launch();
+  if (kSkip && threadIdx.x == 0) {
+    uint32_t mask = 0;
+    const int s0 = prm.skip_off[0], s1 = prm.skip_off[1];
+    for (int i = s0; i < s1; ++i) mask |= 1u << (prm.skip_ids[i] & 31);
+    sm.skip_mask = mask;
   }
   tc_fence_before();
   __syncthreads();
@@ -291,8 +293,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         const int et = (int)threadIdx.x - 64, col = t.n0 + et;
         const bool in = et < t.w && col < N;
         const float* second = prm.scale ? prm.scale : prm.ln_c;
-        const float v0 = in && prm.bias ? __ldg(prm.bias + col) : 0.f;
-        const float v1 = in && second ? __ldg(second + col) : 0.f;
+        const float v0 = in && prm.bias ? prm.bias[col] : 0.f;
+        const float v1 = in && second ? second[col] : 0.f;
         epi_sync();  // every warp is done with the previous tile's
         if (et < kBN) {
           sm.vec[0][et] = v0;
@@ -310,7 +312,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       if (prm.ln_part && row_ok) {
 #pragma unroll
         for (int b = 0; b < 4; ++b)
-          if (2 * b < nb) lnp[b] = __ldg(lpp + b);
+          if (2 * b < nb) lnp[b] = lpp[b];
       }
       const bool ok = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, prm.err, abort_flag);
       if (!ok) break;
@@ -331,7 +333,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         for (int b = 0; b < 4; ++b)
           if (2 * b < nb) sm_ += lnp[b].x + lnp[b].z;
         for (int b = 4; 2 * b < nb; ++b) {
-          const float4 p4 = __ldg(lpp + b);
+          const float4 p4 = lpp[b];
           sm_ += p4.x + p4.z;
         }
         ln_mu = sm_ / (float)nb;
@@ -344,7 +346,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
           }
         }
         for (int b = 4; 2 * b < nb; ++b) {
-          const float4 p4 = __ldg(lpp + b);
+          const float4 p4 = lpp[b];
           const float d0 = p4.x - ln_mu, d1 = p4.z - ln_mu;
           m2 += p4.y + p4.w + 128.f * (d0 * d0 + d1 * d1);
         }
@@ -424,7 +426,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         const float* nbv = is_q ? prm.qn_b : prm.kn_b;
         int py = 0, px = 0;  // the row's position inside its view
         if (prm.rope_cs) {
-          const int tok = prm.tok_index && row_ok ? __ldg(prm.tok_index + row) : row;
+          const int tok = prm.tok_index && row_ok ? prm.tok_index[row] : row;
           const int t = tok % prm.tok_per_view - prm.patch_start;
           if (t >= 0) {
             py = t / prm.grid_w + 1;
@@ -456,8 +458,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
             const float2 nm = make_float2(-mean * rstd, -mean * rstd), rs = make_float2(rstd, rstd);
 #pragma unroll
             for (int q = 0; q < 16; ++q) {
-              const float4 g4 = __ldg(reinterpret_cast<const float4*>(ng) + q);
-              const float4 b4 = __ldg(reinterpret_cast<const float4*>(nbv) + q);
+              const float4 g4 = reinterpret_cast<const float4*>(ng)[q];
+              const float4 b4 = reinterpret_cast<const float4*>(nbv)[q];
               const float2 a0 = ffma2(ffma2(make_float2(x[4 * q], x[4 * q + 1]), rs, nm),
                                       make_float2(g4.x, g4.y), make_float2(b4.x, b4.y));
               const float2 a1 = ffma2(ffma2(make_float2(x[4 * q + 2], x[4 * q + 3]), rs, nm),
@@ -474,7 +476,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
               const float4* cs = reinterpret_cast<const float4*>(prm.rope_cs + (size_t)(ax ? px : py) * 16);
 #pragma unroll
               for (int q = 0; q < 8; ++q) {  // frequencies 2q, 2q + 1: (cos, sin) pairs
-                const float4 t4 = __ldg(cs + q);
+                const float4 t4 = cs[q];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                   const int i = 32 * ax + 2 * q + e;
@@ -594,10 +596,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
 // RoPE angles in double precision: table[p][i] = (cos, sin)(p base^(-i / 16)).
 __global__ void rope_table_kernel(int max_pos, double base, float2* table) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= (max_pos + 1) * 16) return;
   const int p = k >> 4, i = k & 15;
   double sn, cs;
   sincos((double)p * pow(base, -(double)i / 16.0), &sn, &cs);
+  pdl_wait();
+  pdl_launch();
+  if (k >= (max_pos + 1) * 16) return;
   table[k] = make_float2((float)cs, (float)sn);
 }
 
@@ -605,43 +609,30 @@ __global__ void rope_table_kernel(int max_pos, double base, float2* table) {
 
 namespace {
 
-// A warp per output column n of W_O: lane l takes channels 2 l, 2 l + 1 of every mean head.
+// A warp per output column of W_O.
 __global__ void wo_mean_fold_kernel(int D, int H, const __nv_bfloat16* w_o, const float* b_o,
                                     const float* mean_v, const int32_t* head_ids,
                                     const int32_t* offsets, float* bias_out) {
-  const int n = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  const int n = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  pdl_wait();
+  pdl_launch();
   if (n >= D) return;  // whole warps
-  const int m0 = __ldg(offsets), m1 = __ldg(offsets + 1);
-  const __nv_bfloat16* wrow = w_o + (size_t)n * H * 64 + 2 * lane;
-  float acc = 0.f;
-  for (int i = m0; i < m1; ++i) {
-    const int h = __ldg(head_ids + i);
-    const uint32_t w2 = __ldg(reinterpret_cast<const unsigned int*>(wrow + h * 64));
-    // the mean head's row of Y as stored: bf16(mean_v), round to nearest even
-    const float2 mv = __ldg(reinterpret_cast<const float2*>(mean_v + h * 64) + lane);
-    const uint32_t mu = pack_bf16x2(mv.x, mv.y);
-    acc = fmaf(bf16_lo(mu), bf16_lo(w2), fmaf(bf16_hi(mu), bf16_hi(w2), acc));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if (lane == 0) bias_out[n] = (b_o ? __ldg(b_o + n) : 0.f) + acc;
+  wo_mean_fold_column(n, H, w_o, b_o, mean_v, head_ids, offsets[0], offsets[1], bias_out);
 }
 
 }  // namespace
 
 cudaError_t launch_rope_table(int max_pos, float base, float2* table, cudaStream_t st) {
   const int n = (max_pos + 1) * 16;
-  rope_table_kernel<<<(n + 255) / 256, 256, 0, st>>>(max_pos, (double)base, table);
-  return cudaGetLastError();
+  return launch_pdl(rope_table_kernel, dim3((n + 255) / 256), 256, 0, st, max_pos, (double)base, table);
 }
 
 cudaError_t launch_wo_mean_fold(int D, int H, const __nv_bfloat16* w_o, const float* b_o,
                                 const float* mean_v, const int32_t* head_ids,
                                 const int32_t* offsets, float* bias_out, cudaStream_t st) {
   const int threads = 256, blocks = (D * 32 + threads - 1) / threads;
-  wo_mean_fold_kernel<<<blocks, threads, 0, st>>>(D, H, w_o, b_o, mean_v, head_ids, offsets,
-                                                  bias_out);
-  return cudaGetLastError();
+  return launch_pdl(wo_mean_fold_kernel, dim3(blocks), threads, 0, st, D, H, w_o, b_o, mean_v, head_ids,
+                    offsets, bias_out);
 }
 
 cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
@@ -689,9 +680,9 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
     cudaError_t le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (le != cudaSuccess) return le;
     prof_before(VP_KERNEL_GEMM, st);
-    kernel<<<grid, 64 + 32 * epi_warps, smem, st>>>(ta, tb, tb_cut, to, tr, prm);
+    le = launch_pdl(kernel, dim3(grid), 64 + 32 * epi_warps, smem, st, ta, tb, tb_cut, to, tr, prm);
     prof_after(st);
-    return cudaGetLastError();
+    return le;
   };
   // Sixteen epilogue warps (64 columns of a row per thread, one staging block each) where the
   // epilogue is what a tile waits for: GELU (137,400 x 4,096 from K = 1,024: 668 us with eight

@@ -28,10 +28,10 @@ __device__ __forceinline__ void broadcast_rows(const HeadAttnArgs& a, const floa
   const int part = tid & 7, rg = tid >> 3;
   const float* mv = vec + 8 * part;
   uint4 val;
-  val.x = pack_bf16x2(__ldg(mv + 0), __ldg(mv + 1));
-  val.y = pack_bf16x2(__ldg(mv + 2), __ldg(mv + 3));
-  val.z = pack_bf16x2(__ldg(mv + 4), __ldg(mv + 5));
-  val.w = pack_bf16x2(__ldg(mv + 6), __ldg(mv + 7));
+  val.x = pack_bf16x2(*(mv + 0), *(mv + 1));
+  val.y = pack_bf16x2(*(mv + 2), *(mv + 3));
+  val.z = pack_bf16x2(*(mv + 4), *(mv + 5));
+  val.w = pack_bf16x2(*(mv + 6), *(mv + 7));
   const int r1 = min(a.N, r0 + kRows);
   for (int row = r0 + rg; row < r1; row += kThreads / 8)
     *reinterpret_cast<uint4*>(a.y + ((size_t)row * a.H + h) * 64 + 8 * part) = val;
@@ -40,13 +40,14 @@ __device__ __forceinline__ void broadcast_rows(const HeadAttnArgs& a, const floa
 __global__ void __launch_bounds__(kThreads, 3) broadcast_heads_kernel(HeadAttnArgs a) {
   __shared__ int s_item;
   const int tid = threadIdx.x;
-  const int s_first = __ldg(a.offsets + 1), m_first = __ldg(a.offsets + 0);
-  const int n_surr = __ldg(a.offsets + 2) - s_first;
+  const int s_first = a.offsets[1], m_first = a.offsets[0];
+  const int n_surr = a.offsets[2] - s_first;
   const int n_mean = s_first - m_first;
   const int chunks = (a.N + kRows - 1) / kRows;
   // Surrogate heads are broadcast rows only without the token-wise correction.
   const int s_items = (a.variant & VP_VARIANT_NO_RESIDUAL) ? n_surr * chunks : 0;
   const int items = s_items + (a.skip_mean_y ? 0 : n_mean * chunks);
+  pdl_launch();
   // Items (surrogate rows head-major, then mean rows) from a counter, so that CTAs started
   // early (on SMs freed early) do more of them.
   for (;;) {
@@ -57,29 +58,30 @@ __global__ void __launch_bounds__(kThreads, 3) broadcast_heads_kernel(HeadAttnAr
     if (it >= items) break;
     if (it < s_items) {
       const int slot = it / chunks, chunk = it - slot * chunks;
-      const int h = __ldg(a.head_ids + s_first + slot);
+      const int h = a.head_ids[s_first + slot];
       broadcast_rows(a, a.ctx + h * 64, h, chunk * kRows, tid);
     } else {
       const int it2 = it - s_items;
       const int slot = it2 / chunks, chunk = it2 - slot * chunks;
-      const int h = __ldg(a.head_ids + m_first + slot);
+      const int h = a.head_ids[m_first + slot];
       broadcast_rows(a, a.mean_v + h * 64, h, chunk * kRows, tid);
     }
   }
   // Do not complete before the full-attention grid: later work in the stream reads all of Y.
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
 }
 
 }  // namespace
 
 cudaError_t launch_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(a.cheap_counter, 0, sizeof(unsigned int), st);
-  if (e != cudaSuccess) return e;
-  e = cudaMemsetAsync(a.fa_count, 0, sizeof(unsigned int) * kFaCountWords, st);
-  if (e != cudaSuccess) return e;
-  if (a.s_attn) {  // 0 for the heads that are not in full mode; full heads max into it
-    e = cudaMemsetAsync(a.s_attn, 0, sizeof(float) * a.H, st);
+  cudaError_t e = cudaSuccess;
+  if (!a.counters_zeroed) {
+    e = cudaMemsetAsync(a.fa_count, 0, sizeof(unsigned int) * kFaCountWords, st);
     if (e != cudaSuccess) return e;
+    if (a.s_attn) {  // 0 for the heads that are not in full mode; full heads max into it
+      e = cudaMemsetAsync(a.s_attn, 0, sizeof(float) * a.H, st);
+      if (e != cudaSuccess) return e;
+    }
   }
   if (a.variant & VP_VARIANT_LINEAR_ATTENTION) {
     // The surrogate heads in linear-attention form, state then apply, before the
@@ -103,17 +105,7 @@ cudaError_t launch_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(3 * num_sms);
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  e = cudaLaunchKernelEx(&cfg, broadcast_heads_kernel, a);
+  e = launch_pdl(broadcast_heads_kernel, dim3(3 * num_sms), kThreads, 0, st, a);
   prof_extra_launch();
   prof_after(st);
   if (e != cudaSuccess) return e;

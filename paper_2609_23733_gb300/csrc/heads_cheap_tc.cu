@@ -115,14 +115,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
   volatile int* abort_flag = &sm.abort_flag;
   unsigned int* err = a.err;
   const int H = a.H;
-  const int m_first = __ldg(a.offsets + 0), s_first = __ldg(a.offsets + 1);
-  const int n_surr = __ldg(a.offsets + 2) - s_first, n_mean = s_first - m_first;
+  const int m_first = a.offsets[0], s_first = a.offsets[1];
+  const int n_surr = a.offsets[2] - s_first, n_mean = s_first - m_first;
   const int T = (a.N + kTcTile - 1) / kTcTile;
   const int surr_items = n_surr * T;
   const int Tm = (a.N + kMeanRows - 1) / kMeanRows;  // mean items per head
   // Mean heads folded into W_O's bias (skip_mean_y) need no rows of Y.
   const int items = surr_items + (a.skip_mean_y ? 0 : n_mean * Tm);
 
+  pdl_launch();
   if (tid == 0) {
     for (int s = 0; s < kTcStages; ++s) {
       mbar_init(&sm.full[s], 1);
@@ -149,18 +150,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     tmem_alloc(&sm.tmem_base, kTcTmemCols);
     tmem_relinquish();
   }
+  // The mean heads folded into W_O's bias (launch_wo_mean_fold's arithmetic), a warp per output
+  // column: a launch of its own between the router and the heads cost 4-5 us a layer.
+  if (a.wo_bias) {
+    for (int n = (int)blockIdx.x * (kTcThreads / 32) + warp; n < H * 64; n += (int)gridDim.x * (kTcThreads / 32))
+      wo_mean_fold_column(n, H, a.w_o, a.b_o, a.mean_v, a.head_ids, m_first, s_first, a.wo_bias);
+  }
   // The surrogate heads' per-head vectors: the first layer's context half folded into c1 (one
   // 64-term dot product per hidden unit), the second layer's biases, C_h.
   for (int i = tid; i < n_surr * 128; i += kTcThreads) {
     const int slot = i >> 7, u = i & 127, uu = u & 63;
-    const int h = __ldg(a.head_ids + s_first + slot);
+    const int h = a.head_ids[s_first + slot];
     const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
     const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
     float acc = __ldg((u < 64 ? a.sw.g1_b : a.sw.d1_b) + h * 64 + uu);
 #pragma unroll
     for (int kq = 0; kq < 8; ++kq) {
       const uint4 wv = __ldg(reinterpret_cast<const uint4*>(w) + kq);
-      const float4 c0 = __ldg(ctx + 2 * kq), c1 = __ldg(ctx + 2 * kq + 1);
+      const float4 c0 = ctx[2 * kq], c1 = ctx[2 * kq + 1];
       acc = fmaf(bf16_lo(wv.x), c0.x, fmaf(bf16_hi(wv.x), c0.y, acc));
       acc = fmaf(bf16_lo(wv.y), c0.z, fmaf(bf16_hi(wv.y), c0.w, acc));
       acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
@@ -169,7 +176,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     sm.c1[slot][u] = acc;
     const float b = __ldg((u < 64 ? a.sw.g2_b : a.sw.d2_b) + h * 64 + uu);
     sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
-    if (u < 64) sm.cx[slot][u] = __ldg(a.ctx + h * 64 + u);
+    if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
   }
   tc_fence_before();
   __syncthreads();
@@ -205,7 +212,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
       }
       if (it < surr_items) {
         const int slot = it / T, tile = it - slot * T;
-        const int h = __ldg(a.head_ids + s_first + slot);
+        const int h = a.head_ids[s_first + slot];
         if (h != cur_h) {  // this head's weights into the next slot
           ++fill;
           cur_h = h;
@@ -234,7 +241,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
         tma_k[st] = k;
       } else {
         const int slot = (it - surr_items) / Tm;
-        const int h = __ldg(a.head_ids + m_first + slot);
+        const int h = a.head_ids[m_first + slot];
         if (elect_one()) {
           sm.stage_item[st] = it;
           sm.stage_fill[st] = -1;
@@ -502,8 +509,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
         if (!ok) break;
         if (gt == 0) mbar_arrive(&sm.taken[g]);  // every thread has read this tile's item
         const int jc = gt & 7;
-        const float4 m0 = __ldg(reinterpret_cast<const float4*>(a.mean_v + h * 64) + 2 * jc);
-        const float4 m1 = __ldg(reinterpret_cast<const float4*>(a.mean_v + h * 64) + 2 * jc + 1);
+        const float4 m0 = reinterpret_cast<const float4*>(a.mean_v + h * 64)[2 * jc];
+        const float4 m1 = reinterpret_cast<const float4*>(a.mean_v + h * 64)[2 * jc + 1];
         const uint4 val = make_uint4(pack_bf16x2(m0.x, m0.y), pack_bf16x2(m0.z, m0.w),
                                      pack_bf16x2(m1.x, m1.y), pack_bf16x2(m1.z, m1.w));
         for (int r = gt >> 3; r < kMeanRows; r += kGroupThreads / 8) {
@@ -572,7 +579,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     tmem_dealloc(tmem, kTcTmemCols);
   }
   // Do not complete before the full-attention grid: later work in the stream reads all of Y.
-  if (tid == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (tid == 0) pdl_wait();
 }
 
 }  // namespace
@@ -597,17 +604,7 @@ cudaError_t launch_cheap_heads_tc(const HeadAttnArgs& a, int num_sms, cudaStream
   if ((e = cudaFuncSetAttribute(cheap_heads_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 smem)) != cudaSuccess)
     return e;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(num_sms);
-  cfg.blockDim = dim3(kTcThreads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, cheap_heads_tc_kernel, maps, a);
+  return launch_pdl(cheap_heads_tc_kernel, dim3(num_sms), kTcThreads, smem, st, maps, a);
 }
 
 }  // namespace vp

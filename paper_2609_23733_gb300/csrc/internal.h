@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <utility>
+
 #include "vp.h"
 
 namespace vp {
@@ -23,7 +25,7 @@ constexpr int kKeyPartial = 2 + 2 * kHeadDim;       // (max, sum, sum p v[64], s
 // Router scratch carved from the caller's workspace (all device pointers).
 struct RouterScratch {
   unsigned int* err;            // device error word (first 256 bytes of the workspace)
-  unsigned int* counters;       // [2 * kMaxHeads + 2] last-CTA counters, zeroed per call
+  unsigned int* counters;       // [2 * kMaxHeads + 2] last-CTA counters, zeroed by the pooling
   float* pool_part;             // [H][kPoolSplitMax][kPoolPartial]
   float* key_part;              // [H][kKeySplitMax][kKeyPartial]
   float* q_pool;                // [H][64]
@@ -34,11 +36,10 @@ struct RouterScratch {
   float* mean_v;                // [H][64]
   int32_t* head_ids;            // [H]
   int32_t* offsets;             // [4]
-  unsigned int* cheap_counter;  // work counter of the cheap head modes
   float* lin_state;             // [H][kLinState] linear-attention state (after the router part)
   float* fa_part;               // split-tail partial O, kFaPartFloats (layout: attn_full.cu)
   float* fa_stats;              // its (m, l, xmax, -) rows, kFaStatsFloats
-  unsigned int* fa_count;       // [kFaTailUnits][4 chains][4 quarters] split arrivals
+  unsigned int* fa_count;       // kFaCountWords: split arrivals, then the counters named below
   float* wo_bias;               // [kMaxHeads * 64] W_O bias with the mean heads folded in
 };
 
@@ -49,6 +50,8 @@ constexpr int kFaTailUnits = 512;
 constexpr size_t kFaPartFloats = (size_t)kFaTailUnits * 4 * 128 * 64;
 constexpr size_t kFaStatsFloats = (size_t)kFaTailUnits * 4 * 128 * 4;
 constexpr size_t kFaCountWords = (size_t)kFaTailUnits * 4 * 4;
+// The last words of that scratch count the split parts and the cheap-head items handed out.
+constexpr size_t kFaUnitCounter = kFaCountWords - 1, kCheapCounter = kFaCountWords - 2;
 
 // Linear-attention state of one head (the §5 compute-mode ablation): S_h [64 c][64 e] =
 // sum_j phi(k_j)[c] v_j[e], then z_h [64] = sum_j phi(k_j), fp32.
@@ -82,6 +85,11 @@ struct RouterArgs {
   const float* bU;
   const float* beta;
   const int32_t* force_modes;
+  // Counters of the head modes that the router clears on its way (a layer's heads run behind it):
+  // zero_words words from zero, and s_attn_zero [H]; NULL: none.
+  unsigned int* zero;
+  int zero_words;
+  float* s_attn_zero;
   // Outputs (NULL = do not copy out); the scratch copies are always written.
   float* s_out;
   int32_t* modes_out;
@@ -125,10 +133,16 @@ struct HeadAttnArgs {
   float* lin_state;             // [H][kLinState] (VP_VARIANT_LINEAR_ATTENTION only)
   float* fa_part;               // split-tail scratch of the full-attention kernel
   float* fa_stats;
-  unsigned int* fa_count;       // zeroed by the launcher
+  unsigned int* fa_count;       // zeroed by launch_heads, or before it (counters_zeroed)
   unsigned int* err;
-  unsigned int* cheap_counter;  // one word of scratch, zeroed by the launcher
+  unsigned int* cheap_counter;  // fa_count[kCheapCounter]
+  int counters_zeroed;          // 1: fa_count and s_attn were cleared earlier in the stream
   int skip_mean_y;              // 1: the mean heads' rows of Y are not written (folded into W_O)
+  // The mean heads folded into W_O's bias by the cheap-heads kernel (see launch_wo_mean_fold):
+  // wo_bias[n], n < 64 H, from W_O and b_O (NULL: 0); wo_bias NULL: not here.
+  const __nv_bfloat16* w_o;
+  const float* b_o;
+  float* wo_bias;
 };
 
 // Full-mode heads (attn_full.cu).
@@ -198,12 +212,13 @@ cudaError_t launch_wo_mean_fold(int D, int H, const __nv_bfloat16* w_o, const fl
 cudaError_t launch_ln_partials(int M, int D, const __nv_bfloat16* x, float2* part, cudaStream_t st);
 // The folded LayerNorm's weights for a projection W [Nout][K] (nn.Linear layout):
 // Wp = W diag(g) (bf16), c[o] = sum_k Wp[o][k] (of the bf16 Wp), bp[o] = b[o] + sum_k W[o][k] beta[k]
-// (b NULL: 0).  K % 256 == 0, K <= 4096.
+// (b NULL: 0).  K % 256 == 0, K <= 4096.  weights_ready: no kernel just before writes W, g, beta or b,
+// and none reads the outputs any more (see ln_fold_kernel).
 // cos / sin of p * base^(-i / 16), p = 0 .. max_pos, i = 0 .. 15: table [max_pos + 1][16].
 cudaError_t launch_rope_table(int max_pos, float base, float2* table, cudaStream_t st);
 cudaError_t launch_ln_fold_weights(int Nout, int K, const __nv_bfloat16* W, const float* g,
                                    const float* beta, const float* b, __nv_bfloat16* Wp,
-                                   float* c, float* bp, cudaStream_t st);
+                                   float* c, float* bp, bool weights_ready, cudaStream_t st);
 
 // Token merging around a block's attention (merge.cu, vp_merge_options).
 struct MergeGeo {
@@ -279,6 +294,25 @@ cudaError_t make_tmap_bf16_2d(CUtensorMap* map, const void* base, uint64_t cols,
 void prof_before(int kind, cudaStream_t st);
 void prof_after(cudaStream_t st);
 void prof_extra_launch();  // one more kernel inside the current bracket
+
+// Launch with programmatic stream serialization: the kernel may start before the one before it
+// in the stream has completed and calls pdl_wait (common.cuh) before it touches what that one
+// reads or writes.
+template <typename... K, typename... A>
+cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                       A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 
 int device_sm_count();
 bool device_is_sm103();

@@ -23,14 +23,16 @@ __global__ void __launch_bounds__(256) layernorm_kernel(int M, const __nv_bfloat
   const int lane = threadIdx.x & 31;
   const int warp_global = blockIdx.x * 8 + (threadIdx.x >> 5);
   const int n_warps = gridDim.x * 8;
+  pdl_wait();
+  pdl_launch();
   float gr[kKeep ? 8 * C : 1], br[kKeep ? 8 * C : 1];
 #pragma unroll
   for (int c = 0; c < (kKeep ? C : 0); ++c) {
     const int col = (c * 32 + lane) * 8;
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(g + col));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(g + col) + 1);
-    const float4 b0 = __ldg(reinterpret_cast<const float4*>(b + col));
-    const float4 b1 = __ldg(reinterpret_cast<const float4*>(b + col) + 1);
+    const float4 g0 = reinterpret_cast<const float4*>(g + col)[0];
+    const float4 g1 = reinterpret_cast<const float4*>(g + col)[1];
+    const float4 b0 = reinterpret_cast<const float4*>(b + col)[0];
+    const float4 b1 = reinterpret_cast<const float4*>(b + col)[1];
     gr[8 * c + 0] = g0.x; gr[8 * c + 1] = g0.y; gr[8 * c + 2] = g0.z; gr[8 * c + 3] = g0.w;
     gr[8 * c + 4] = g1.x; gr[8 * c + 5] = g1.y; gr[8 * c + 6] = g1.z; gr[8 * c + 7] = g1.w;
     br[8 * c + 0] = b0.x; br[8 * c + 1] = b0.y; br[8 * c + 2] = b0.z; br[8 * c + 3] = b0.w;
@@ -44,7 +46,7 @@ __global__ void __launch_bounds__(256) layernorm_kernel(int M, const __nv_bfloat
       const int row = min(r0 + k, M - 1);
 #pragma unroll
       for (int c = 0; c < C; ++c)
-        u[k][c] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)row * D + (c * 32 + lane) * 8));
+        u[k][c] = *reinterpret_cast<const uint4*>(x + (size_t)row * D + (c * 32 + lane) * 8);
     }
 #pragma unroll
     for (int k = 0; k < kRows; ++k) {
@@ -84,10 +86,10 @@ __global__ void __launch_bounds__(256) layernorm_kernel(int M, const __nv_bfloat
             for (int e = 0; e < 8; ++e) y[e] = (v[8 * c + e] - mean) * rstd * gr[8 * c + e] + br[8 * c + e];
           } else {
             const int col = (c * 32 + lane) * 8;
-            const float4 g0 = __ldg(reinterpret_cast<const float4*>(g + col));
-            const float4 g1 = __ldg(reinterpret_cast<const float4*>(g + col) + 1);
-            const float4 b0 = __ldg(reinterpret_cast<const float4*>(b + col));
-            const float4 b1 = __ldg(reinterpret_cast<const float4*>(b + col) + 1);
+            const float4 g0 = reinterpret_cast<const float4*>(g + col)[0];
+            const float4 g1 = reinterpret_cast<const float4*>(g + col)[1];
+            const float4 b0 = reinterpret_cast<const float4*>(b + col)[0];
+            const float4 b1 = reinterpret_cast<const float4*>(b + col)[1];
             const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
             const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
@@ -116,11 +118,13 @@ __global__ void __launch_bounds__(256) ln_partials_kernel(int M, const __nv_bflo
   constexpr int D = 256 * C;
   const int lane = threadIdx.x & 31;
   const int n_warps = gridDim.x * 8;
+  pdl_wait();
+  pdl_launch();
   for (int row = blockIdx.x * 8 + (threadIdx.x >> 5); row < M; row += n_warps) {
     uint4 u[C];
 #pragma unroll
     for (int c = 0; c < C; ++c)
-      u[c] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)row * D + (c * 32 + lane) * 8));
+      u[c] = *reinterpret_cast<const uint4*>(x + (size_t)row * D + (c * 32 + lane) * 8);
 #pragma unroll
     for (int c = 0; c < C; ++c) {
       const uint32_t w[4] = {u[c].x, u[c].y, u[c].z, u[c].w};
@@ -152,25 +156,33 @@ __global__ void __launch_bounds__(256) ln_partials_kernel(int M, const __nv_bflo
 }
 
 // Folded LayerNorm weights: one warp per output row o of W [Nout][K]; lane l holds the
-// 16-byte chunks c 32 + l of the row.
+// 16-byte chunks c 32 + l of the row.  With weights_ready W is a weight (not another kernel's
+// output) and the outputs' last readers have completed when the kernel may start (every kernel
+// lets the next one start after its own wait): it then runs beside the kernel before it (the
+// previous block's FFN-down) and waits only at its end.
 template <int C>
 __global__ void __launch_bounds__(256) ln_fold_kernel(int Nout, const __nv_bfloat16* W,
                                                       const float* g, const float* beta,
                                                       const float* b, __nv_bfloat16* Wp,
-                                                      float* cs, float* bp) {
+                                                      float* cs, float* bp, bool weights_ready) {
   constexpr int K = 256 * C;
   const int lane = threadIdx.x & 31;
   const int o = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (o >= Nout) return;
+  if (!weights_ready) pdl_wait();
+  pdl_launch();
+  if (o >= Nout) {
+    if (weights_ready) pdl_wait();
+    return;
+  }
   float csum = 0.f, bsum = 0.f;
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int k0 = (c * 32 + lane) * 8;
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(W + (size_t)o * K + k0));
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(g + k0));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(g + k0) + 1);
-    const float4 e0 = __ldg(reinterpret_cast<const float4*>(beta + k0));
-    const float4 e1 = __ldg(reinterpret_cast<const float4*>(beta + k0) + 1);
+    const uint4 u = reinterpret_cast<const uint4*>(W + (size_t)o * K + k0)[0];
+    const float4 g0 = reinterpret_cast<const float4*>(g + k0)[0];
+    const float4 g1 = reinterpret_cast<const float4*>(g + k0)[1];
+    const float4 e0 = reinterpret_cast<const float4*>(beta + k0)[0];
+    const float4 e1 = reinterpret_cast<const float4*>(beta + k0)[1];
     const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     const float ee[8] = {e0.x, e0.y, e0.z, e0.w, e1.x, e1.y, e1.z, e1.w};
     const uint32_t w[4] = {u.x, u.y, u.z, u.w};
@@ -194,6 +206,7 @@ __global__ void __launch_bounds__(256) ln_fold_kernel(int Nout, const __nv_bfloa
     cs[o] = csum;
     bp[o] = (b ? b[o] : 0.f) + bsum;
   }
+  if (weights_ready) pdl_wait();
 }
 
 }  // namespace
@@ -204,36 +217,38 @@ cudaError_t launch_ln_partials(int M, int D, const __nv_bfloat16* x, float2* par
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int blocks = max(1, min((M + 7) / 8, sms * 8));
+  cudaError_t e;
   prof_before(VP_KERNEL_LAYER_NORM, st);
   switch (D / 256) {
-    case 1: ln_partials_kernel<1><<<blocks, 256, 0, st>>>(M, x, part); break;
-    case 2: ln_partials_kernel<2><<<blocks, 256, 0, st>>>(M, x, part); break;
-    case 3: ln_partials_kernel<3><<<blocks, 256, 0, st>>>(M, x, part); break;
-    case 4: ln_partials_kernel<4><<<blocks, 256, 0, st>>>(M, x, part); break;
-    case 8: ln_partials_kernel<8><<<blocks, 256, 0, st>>>(M, x, part); break;
-    case 16: ln_partials_kernel<16><<<blocks, 256, 0, st>>>(M, x, part); break;
+    case 1: e = launch_pdl(ln_partials_kernel<1>, dim3(blocks), 256, 0, st, M, x, part); break;
+    case 2: e = launch_pdl(ln_partials_kernel<2>, dim3(blocks), 256, 0, st, M, x, part); break;
+    case 3: e = launch_pdl(ln_partials_kernel<3>, dim3(blocks), 256, 0, st, M, x, part); break;
+    case 4: e = launch_pdl(ln_partials_kernel<4>, dim3(blocks), 256, 0, st, M, x, part); break;
+    case 8: e = launch_pdl(ln_partials_kernel<8>, dim3(blocks), 256, 0, st, M, x, part); break;
+    case 16: e = launch_pdl(ln_partials_kernel<16>, dim3(blocks), 256, 0, st, M, x, part); break;
     default: prof_after(st); return cudaErrorInvalidValue;
   }
   prof_after(st);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_ln_fold_weights(int Nout, int K, const __nv_bfloat16* W, const float* g,
                                    const float* beta, const float* b, __nv_bfloat16* Wp,
-                                   float* c, float* bp, cudaStream_t st) {
+                                   float* c, float* bp, bool weights_ready, cudaStream_t st) {
   const int blocks = (Nout + 7) / 8;
+  cudaError_t e;
   prof_before(VP_KERNEL_LAYER_NORM, st);
   switch (K / 256) {
-    case 1: ln_fold_kernel<1><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
-    case 2: ln_fold_kernel<2><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
-    case 3: ln_fold_kernel<3><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
-    case 4: ln_fold_kernel<4><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
-    case 8: ln_fold_kernel<8><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
-    case 16: ln_fold_kernel<16><<<blocks, 256, 0, st>>>(Nout, W, g, beta, b, Wp, c, bp); break;
+    case 1: e = launch_pdl(ln_fold_kernel<1>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
+    case 2: e = launch_pdl(ln_fold_kernel<2>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
+    case 3: e = launch_pdl(ln_fold_kernel<3>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
+    case 4: e = launch_pdl(ln_fold_kernel<4>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
+    case 8: e = launch_pdl(ln_fold_kernel<8>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
+    case 16: e = launch_pdl(ln_fold_kernel<16>, dim3(blocks), 256, 0, st, Nout, W, g, beta, b, Wp, c, bp, weights_ready); break;
     default: prof_after(st); return cudaErrorInvalidValue;
   }
   prof_after(st);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_layer_norm(int M, int D, const __nv_bfloat16* x, const float* g,
@@ -243,18 +258,19 @@ cudaError_t launch_layer_norm(int M, int D, const __nv_bfloat16* x, const float*
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int blocks = max(1, min((M + 15) / 16, sms * 4));
+  cudaError_t e;
   prof_before(VP_KERNEL_LAYER_NORM, st);
   switch (D / 256) {
-    case 1: layernorm_kernel<1><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
-    case 2: layernorm_kernel<2><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
-    case 3: layernorm_kernel<3><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
-    case 4: layernorm_kernel<4><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
-    case 8: layernorm_kernel<8><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
-    case 16: layernorm_kernel<16><<<blocks, 256, 0, st>>>(M, x, g, b, eps, out); break;
+    case 1: e = launch_pdl(layernorm_kernel<1>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
+    case 2: e = launch_pdl(layernorm_kernel<2>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
+    case 3: e = launch_pdl(layernorm_kernel<3>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
+    case 4: e = launch_pdl(layernorm_kernel<4>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
+    case 8: e = launch_pdl(layernorm_kernel<8>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
+    case 16: e = launch_pdl(layernorm_kernel<16>, dim3(blocks), 256, 0, st, M, x, g, b, eps, out); break;
     default: prof_after(st); return cudaErrorInvalidValue;
   }
   prof_after(st);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace vp

@@ -710,7 +710,7 @@ cudaError_t launch_merge_prepare(const MergeGeo& g, int H, const __nv_bfloat16* 
   if (e != cudaSuccess) return e;
   // The metric of LN1(x) with LN1 folded into its weights, as in the QKV projection.
   if ((e = launch_ln_fold_weights(64, D, s.wbar, ln.g, ln.b, s.bbar, ln.w_fold, ln.c_fold,
-                                  ln.b_fold, st)) != cudaSuccess)
+                                  ln.b_fold, false, st)) != cudaSuccess)
     return e;
   LinearArgs la{};
   la.M = g.N;

@@ -4,10 +4,11 @@
 //   router_pool_tc_kernel  (§4.1, pooling): e_i = w_h^T (tanh(W_h q_i + bW) (.) sigma(U_h q_i + bU))
 //       The [128 tokens x 64] x [64 x 128] projection onto [W_h; U_h] runs on the
 //       tcgen05 tensor cores (TMA-fed shared-memory operands, fp32 accumulators in TMEM);
-//       each token thread keeps a running (max, sum, sum p q) of alpha's softmax, the CTA
-//       merges them, and the last CTA of a head combines the partials into
-//       q_pool = sum_i alpha_i q_i.
+//       each token thread keeps a running (max, sum, sum p q) of alpha's softmax and the CTA
+//       merges them into a partial.
 //   router_keys_kernel  (§4.1 routing attention + §4.3 context + mean of V):
+//       every CTA combines its head's partials into q_pool = sum_i alpha_i q_i (a few KB from
+//       L2, against a counter, a fence and a serial combine at the end of the pooling);
 //       l_j = beta_h / sqrt(d) * q_pool . k_j; running (max, sum 2^(l-max), sum p v, sum v)
 //       per CTA; the last CTA of a head derives s_h = max_j r_h(j) = 1 / sum_j e^(l_j - max),
 //       C_h = r_h V_h and mean_v, applies the routing equation (§4.2), and the last head
@@ -58,36 +59,6 @@ __device__ __forceinline__ void token_range(int N, int n_split, int split, int a
   t1 = min(N, t0 + per);
 }
 
-// The last CTA of head h to publish its partial (max, sum, sum p q) combines the n_split
-// partials into q_pool.  Called by every thread of the CTA.
-__device__ __forceinline__ void pool_finish(const RouterArgs& a, const RouterScratch& sc, int h,
-                                            int n_split) {
-  __shared__ int s_last;
-  const int tid = threadIdx.x;
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&sc.counters[h], 1u) == (unsigned)(n_split - 1));
-  __syncthreads();
-  if (!s_last) return;
-  __threadfence();
-  if (tid < 64) {
-    const float* pp = sc.pool_part + (size_t)h * kPoolSplitMax * kPoolPartial;
-    float Mx = -INFINITY;
-    for (int s = 0; s < n_split; ++s) Mx = fmaxf(Mx, __ldcg(pp + s * kPoolPartial));
-    float acc = 0.f, l = 0.f;
-    for (int s = 0; s < n_split; ++s) {
-      const float ms = __ldcg(pp + s * kPoolPartial);
-      if (ms == -INFINITY) continue;
-      const float f = __expf(ms - Mx);
-      l += f * __ldcg(pp + s * kPoolPartial + 1);
-      acc += f * __ldcg(pp + s * kPoolPartial + 2 + tid);
-    }
-    const float q = acc / l;
-    sc.q_pool[h * 64 + tid] = q;
-    if (a.q_pool_out) a.q_pool_out[h * 64 + tid] = q;
-  }
-}
-
 // ------------------------------------------------------------------ pooling sweep (tcgen05)
 // The same sweep with the [W_h; U_h] projection on the 5th-generation tensor cores: a CTA
 // takes a run of 128-token tiles of one head.
@@ -100,7 +71,8 @@ __device__ __forceinline__ void pool_finish(const RouterArgs& a, const RouterScr
 //            softmax of its own tokens (max M, sum, sum p q over the 64 channels of its Q row,
 //            read from the shared-memory tile; rescaled only when M grows), released tile by
 //            tile; at the end the 128 threads' partials merge into the CTA's (max, sum,
-//            sum p q), which pool_finish combines over the CTAs of the head.
+//            sum p q).
+// The counters of the kernels behind it are cleared here.
 constexpr int kPoolTcStages = 4;
 constexpr int kPoolTcThreads = 192;
 constexpr int kPoolAccBufs = 2;    // 128-column fp32 accumulators per CTA
@@ -160,14 +132,23 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
     fence_proxy_async_smem();
     tma_prefetch_desc(&tmap_q);
   }
+  if (warp == 5) {
+    tmem_alloc(&sm.tmem_base, kPoolTcTmemCols);
+    tmem_relinquish();
+  }
+  pdl_wait();
+  pdl_launch();
+  {  // counters of the key sweep, and of the head modes where they follow
+    const int cta = blockIdx.y * gridDim.x + blockIdx.x, step = gridDim.x * gridDim.y * kPoolTcThreads;
+    if (cta == 0 && tid < 128) sc.counters[tid] = 0u;
+    if (a.zero)
+      for (int i = cta * kPoolTcThreads + tid; i < a.zero_words; i += step) a.zero[i] = 0u;
+    if (a.s_attn_zero && cta == 0 && tid < a.H) a.s_attn_zero[tid] = 0.f;
+  }
   if (tid < 64) {
     sm.bias[tid] = a.bW ? a.bW[h * 64 + tid] : 0.f;
     sm.bias[64 + tid] = a.bU ? a.bU[h * 64 + tid] : 0.f;
     sm.wv[tid] = __bfloat162float(a.w[h * 64 + tid]);
-  }
-  if (warp == 5) {
-    tmem_alloc(&sm.tmem_base, kPoolTcTmemCols);
-    tmem_relinquish();
   }
   tc_fence_before();
   __syncthreads();
@@ -349,7 +330,6 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
     tc_fence_after();
     tmem_dealloc(tmem, kPoolTcTmemCols);
   }
-  pool_finish(a, sc, h, n_split);
 }
 
 // ------------------------------------------------------------------ key sweep
@@ -374,8 +354,24 @@ __device__ void bin_heads_warp(int H, const int32_t* modes, int32_t* head_ids, i
   if (lane == 0) offsets[3] = base;
 }
 
+// A CTA's row-group sums, or a head's partials once they are combined (never both).
+union KeySmem {
+  struct {
+    float m[32], l[32];
+    float acc[32][64], sum[32][64];
+  } rows;
+  float pool[kPoolSplitMax * kPoolPartial];
+  float part[kKeySplitMax * kKeyPartial];
+};
+
+// n floats of another CTA's making (L2) into shared memory by the whole CTA, all loads in flight.
+__device__ __forceinline__ void stage_floats(float* dst, const float* src, int n) {
+#pragma unroll 8
+  for (int i = threadIdx.x; i < n; i += kKeyThreads) dst[i] = __ldcg(src + i);
+}
+
 __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, RouterScratch sc,
-                                                                   int n_split) {
+                                                                   int pool_split, int n_split) {
   const int h = blockIdx.y, split = blockIdx.x;
   const int N = a.N, H = a.H;
   const size_t row_pitch = (size_t)3 * H * kHeadDim;
@@ -385,34 +381,62 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
   const float kLog2e = 1.4426950408889634f;
   const float beta = a.beta ? a.beta[h] : 1.f;
   const float cscale = beta * 0.125f * kLog2e;  // beta / sqrt(64), in log2 units
-  float q[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) q[i] = __ldcg(sc.q_pool + h * 64 + 8 * part + i) * cscale;
-
+  __shared__ KeySmem sk;
+  __shared__ float s_q[64];
+  pdl_wait();
+  pdl_launch();
   int t0, t1;
   token_range(N, n_split, split, 128, t0, t1);
   const __nv_bfloat16* kb = a.qkv + (size_t)(H + h) * kHeadDim + 8 * part;
   const __nv_bfloat16* vb = a.qkv + (size_t)(2 * H + h) * kHeadDim + 8 * part;
-
-  float m = -INFINITY, l = 0.f, accv[8], sumv[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) accv[i] = sumv[i] = 0.f;
-
-  // The loop bound is uniform across the CTA so that the 8-lane shuffles below always
-  // run with the whole warp; rows past t1 are loaded from row t0 and masked.  Four rows per
-  // row group are in flight (eight 16-byte loads per thread) before any arithmetic.
-  // The next batch of rows is loaded while the current one is computed.
+  // Four rows per row group are in flight (eight 16-byte loads per thread) before any
+  // arithmetic, the first ones while q_pool is computed; rows past t1 are loaded from row t0.
   uint4 nk[4], nv[4];
   auto load_batch = [&](int base) {
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       const int row = base + g + 32 * u;
       const size_t o = (size_t)(row < t1 ? row : t0) * row_pitch;
-      nk[u] = __ldg(reinterpret_cast<const uint4*>(kb + o));
-      nv[u] = __ldg(reinterpret_cast<const uint4*>(vb + o));
+      nk[u] = *reinterpret_cast<const uint4*>(kb + o);
+      nv[u] = *reinterpret_cast<const uint4*>(vb + o);
     }
   };
   if (t0 < t1) load_batch(t0);
+  // q_pool from the pooling's partials: threads 0-63, a channel each, splits in order.
+  stage_floats(sk.pool, sc.pool_part + (size_t)h * kPoolSplitMax * kPoolPartial, pool_split * kPoolPartial);
+  __syncthreads();
+  if (tid < 64) {
+    const float* pp = sk.pool;
+    float Mx = -INFINITY;
+    for (int s = 0; s < pool_split; ++s) Mx = fmaxf(Mx, pp[s * kPoolPartial]);
+    float acc = 0.f, l = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < pool_split; ++s) {
+      const float ms = pp[s * kPoolPartial];
+      if (ms == -INFINITY) continue;
+      const float f = __expf(ms - Mx);
+      l += f * pp[s * kPoolPartial + 1];
+      acc += f * pp[s * kPoolPartial + 2 + tid];
+    }
+    const float qp = acc / l;
+    s_q[tid] = qp;
+    if (split == 0) {
+      sc.q_pool[h * 64 + tid] = qp;
+      if (a.q_pool_out) a.q_pool_out[h * 64 + tid] = qp;
+    }
+  }
+  __syncthreads();
+  float q[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) q[i] = s_q[8 * part + i] * cscale;
+
+  float m = -INFINITY, l = 0.f, accv[8], sumv[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) accv[i] = sumv[i] = 0.f;
+
+  // The loop bound is uniform across the CTA so that the 8-lane shuffles below always
+  // run with the whole warp; rows past t1 are masked.  The next batch of rows is loaded while
+  // the current one is computed.
   for (int base = t0; base < t1; base += 128) {
     uint4 kr[4], vr[4];
     bool valid[4];
@@ -453,30 +477,30 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
       }
     }
   }
-  // Combine the 32 row groups of the CTA.
-  __shared__ float s_m[32], s_l[32];
-  __shared__ float s_acc[32][64], s_sum[32][64];
+  // Combine the 32 row groups of the CTA: threads 0-63, a channel each, groups in order.
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    s_acc[g][8 * part + i] = accv[i];
-    s_sum[g][8 * part + i] = sumv[i];
+    sk.rows.acc[g][8 * part + i] = accv[i];
+    sk.rows.sum[g][8 * part + i] = sumv[i];
   }
   if (part == 0) {
-    s_m[g] = m;
-    s_l[g] = l;
+    sk.rows.m[g] = m;
+    sk.rows.l[g] = l;
   }
   __syncthreads();
   float* kp = sc.key_part + ((size_t)h * kKeySplitMax + split) * kKeyPartial;
   if (tid < 64) {
     float Mx = -INFINITY;
-    for (int i = 0; i < 32; ++i) Mx = fmaxf(Mx, s_m[i]);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) Mx = fmaxf(Mx, sk.rows.m[i]);
     float acc = 0.f, sum = 0.f, ll = 0.f;
+#pragma unroll 8
     for (int i = 0; i < 32; ++i) {
-      sum += s_sum[i][tid];
-      if (s_m[i] == -INFINITY) continue;
-      const float f = fast_exp2(s_m[i] - Mx);
-      acc += f * s_acc[i][tid];
-      ll += f * s_l[i];
+      sum += sk.rows.sum[i][tid];
+      if (sk.rows.m[i] == -INFINITY) continue;
+      const float f = fast_exp2(sk.rows.m[i] - Mx);
+      acc += f * sk.rows.acc[i][tid];
+      ll += f * sk.rows.l[i];
     }
     kp[2 + tid] = acc;
     kp[2 + 64 + tid] = sum;
@@ -493,19 +517,23 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
   if (!s_last) return;
   __threadfence();
   // Last CTA of head h: saliency, context, mean of V, mode.
+  stage_floats(sk.part, sc.key_part + (size_t)h * kKeySplitMax * kKeyPartial, n_split * kKeyPartial);
+  __syncthreads();
   if (tid < 64) {
-    const float* pp = sc.key_part + (size_t)h * kKeySplitMax * kKeyPartial;
+    const float* pp = sk.part;
     float Mx = -INFINITY;
-    for (int s = 0; s < n_split; ++s) Mx = fmaxf(Mx, __ldcg(pp + s * kKeyPartial));
+#pragma unroll 4
+    for (int s = 0; s < n_split; ++s) Mx = fmaxf(Mx, pp[s * kKeyPartial]);
     float acc = 0.f, sum = 0.f, ll = 0.f;
+#pragma unroll 4
     for (int s = 0; s < n_split; ++s) {
       const float* q2 = pp + s * kKeyPartial;
-      sum += __ldcg(q2 + 2 + 64 + tid);
-      const float ms = __ldcg(q2);
+      sum += q2[2 + 64 + tid];
+      const float ms = q2[0];
       if (ms == -INFINITY) continue;
       const float f = fast_exp2(ms - Mx);
-      ll += f * __ldcg(q2 + 1);
-      acc += f * __ldcg(q2 + 2 + tid);
+      ll += f * q2[1];
+      acc += f * q2[2 + tid];
     }
     const float ctx = acc / ll;
     const float mv = sum / (float)N;
@@ -549,6 +577,8 @@ __global__ void __launch_bounds__(256) router_r_kernel(RouterArgs a, RouterScrat
   const float kLog2e = 1.4426950408889634f;
   const float beta = a.beta ? a.beta[h] : 1.f;
   const float cscale = beta * 0.125f * kLog2e;
+  pdl_wait();
+  pdl_launch();
   float q[8];
 #pragma unroll
   for (int i = 0; i < 8; ++i) q[i] = __ldcg(sc.q_pool + h * 64 + 8 * part + i) * cscale;
@@ -557,7 +587,7 @@ __global__ void __launch_bounds__(256) router_r_kernel(RouterArgs a, RouterScrat
   for (int base = blockIdx.x * 32; base < N; base += gridDim.x * 32) {  // uniform bound
     const int row = base + g;
     const bool valid = row < N;
-    const uint4 kk = __ldg(reinterpret_cast<const uint4*>(kb + (size_t)(valid ? row : 0) * row_pitch));
+    const uint4 kk = *reinterpret_cast<const uint4*>(kb + (size_t)(valid ? row : 0) * row_pitch);
     const uint32_t kw[4] = {kk.x, kk.y, kk.z, kk.w};
     float dot = 0.f;
 #pragma unroll
@@ -641,7 +671,6 @@ RouterScratch carve_router_scratch(void* ws, int H) {
   p += kMaxHeads * 4;
   sc.head_ids = reinterpret_cast<int32_t*>(p);
   sc.offsets = sc.head_ids + kMaxHeads;
-  sc.cheap_counter = sc.counters + 96;  // counters[0 .. 2 * kMaxHeads] serve the router
   sc.lin_state = reinterpret_cast<float*>(static_cast<char*>(ws) + router_scratch_bytes(H));
   sc.fa_part = sc.lin_state + (size_t)kMaxHeads * kLinState;
   sc.fa_stats = sc.fa_part + kFaPartFloats;
@@ -652,8 +681,7 @@ RouterScratch carve_router_scratch(void* ws, int H) {
 
 cudaError_t launch_router(const RouterArgs& a, const RouterScratch& sc, int num_sms,
                           cudaStream_t st) {
-  cudaError_t e = cudaMemsetAsync(sc.counters, 0, 512, st);
-  if (e != cudaSuccess) return e;
+  cudaError_t e;
   // Pooling sweep on the tensor cores: two CTAs per SM (TMEM 2 x 256 columns), runs of
   // 128-token tiles.
   const int n_tiles = (a.N + 127) / 128;
@@ -671,28 +699,22 @@ cudaError_t launch_router(const RouterArgs& a, const RouterScratch& sc, int num_
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess)
     return e;
   prof_before(VP_KERNEL_ROUTER_POOL, st);
-  if (bias)
-    router_pool_tc_kernel<true><<<dim3(pool_split, a.H), kPoolTcThreads, smem, st>>>(tq, tw, tu, a, sc,
-                                                                                    pool_split);
-  else
-    router_pool_tc_kernel<false><<<dim3(pool_split, a.H), kPoolTcThreads, smem, st>>>(tq, tw, tu, a, sc,
-                                                                                     pool_split);
+  e = launch_pdl(bias ? router_pool_tc_kernel<true> : router_pool_tc_kernel<false>,
+                 dim3(pool_split, a.H), kPoolTcThreads, smem, st, tq, tw, tu, a, sc, pool_split);
   prof_after(st);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   int key_split = (4 * num_sms + a.H - 1) / a.H;
   key_split = max(1, min(min(key_split, kKeySplitMax), (a.N + 255) / 256));
   prof_before(VP_KERNEL_ROUTER_KEYS, st);
-  router_keys_kernel<<<dim3(key_split, a.H), kKeyThreads, 0, st>>>(a, sc, key_split);
+  e = launch_pdl(router_keys_kernel, dim3(key_split, a.H), kKeyThreads, 0, st, a, sc, pool_split,
+                 key_split);
   prof_after(st);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (a.r_out) {
     int blocks = max(1, min((a.N + 31) / 32, (2 * num_sms + a.H - 1) / a.H));
     prof_before(VP_KERNEL_ROUTER_R, st);
-    router_r_kernel<<<dim3(blocks, a.H), 256, 0, st>>>(a, sc);
+    e = launch_pdl(router_r_kernel, dim3(blocks, a.H), 256, 0, st, a, sc);
     prof_after(st);
-    e = cudaGetLastError();
   }
   return e;
 }
