@@ -330,12 +330,14 @@ vp_status run_heads(const vp_dims* dm, const __nv_bfloat16* qkv, const int32_t* 
   ha.lin_state = sc.lin_state;
   ha.fa_part = sc.fa_part;
   ha.fa_stats = sc.fa_stats;
-  ha.fa_count = sc.fa_count;
+  ha.counters = sc.head_counters;
+  ha.attn_ctas = device_sm_count();
   ha.sw = make_surrogate_args(sw);
   ha.y = y;
   ha.s_attn = s_attn;
   ha.err = sc.err;
-  ha.cheap_counter = sc.fa_count + kCheapCounter;
+  ha.cheap_counter = sc.head_counters + kCheapCounter;
+  ha.fold_counter = sc.head_counters + kFoldCounter;
   ha.counters_zeroed = in_layer ? 1 : 0;
   ha.w_o = w_o;
   ha.b_o = b_o;
@@ -387,8 +389,7 @@ vp_status run_layer(const vp_dims* dm, const __nv_bfloat16* xin, const vp_bf16* 
   RouterArgs ra = make_router_args(dm, reinterpret_cast<const vp_bf16*>(qkv), rw, force_modes);
   ra.s_out = s_out;
   ra.modes_out = modes_out;
-  ra.zero = sc.fa_count;
-  ra.zero_words = (int)kFaCountWords;
+  ra.head_counters = sc.head_counters;
   ra.s_attn_zero = s_attn_out;
   VP_TRY(from_cuda(launch_router(ra, sc, sms, st)));
   const __nv_bfloat16* wo = reinterpret_cast<const __nv_bfloat16*>(w_o);

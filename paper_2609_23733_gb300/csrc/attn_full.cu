@@ -33,6 +33,7 @@
 // issuing work, waits (bounded) for its own outstanding copies and MMAs, frees TMEM, exits.
 #include <math.h>
 
+#include "attn_plan.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -40,15 +41,9 @@ namespace vp {
 
 namespace {
 
-#ifndef VP_ATTN_CHAINS
-#define VP_ATTN_CHAINS 3
-#endif
-#ifndef VP_ATTN_BN
-#define VP_ATTN_BN 64
-#endif
-constexpr int kChains = VP_ATTN_CHAINS;  // query tiles (chains) per work item
-constexpr int kBM = 128;                 // query rows per tile
-constexpr int kBN = VP_ATTN_BN;          // keys per tile
+constexpr int kChains = kFaChains;       // query tiles (chains) per work item
+constexpr int kBM = kFaRows;             // query rows per tile
+constexpr int kBN = kFaKeys;             // keys per tile
 constexpr int kStages = 512 / kBN;       // K/V ring depth: 64 KB of K and 64 KB of V
 constexpr int kQTileBytes = kBM * 64 * 2;
 constexpr int kKVTileBytes = kBN * 64 * 2;
@@ -67,11 +62,6 @@ constexpr int kThreads = 128 + 128 * kChains;
 constexpr int kCtrlRegs = kChains == 3 ? 56 : 80;
 constexpr int kSoftRegs = kChains == 3 ? 152 : 208;
 static_assert(128 * kCtrlRegs + 128 * kChains * kSoftRegs <= 65536, "register split");
-
-struct Plan {
-  int R, T, S, units;
-  int whole;  // units of the whole-group instance (they come first)
-};
 
 // Units announced by the producer of a split-parts CTA.  Four slots: the MMA warps run at most one
 // tile ahead of the softmax and the producer at most two units ahead of the MMA warps, so slot
@@ -100,80 +90,17 @@ struct FullParams {
   const int32_t* offsets;
   __nv_bfloat16* y;
   float* s_attn;  // [H] MaxAttn saliency (zeroed by the launcher), or NULL
-  float* part;    // split-tail partial O, (m, l, xmax) and arrival counters (zeroed)
+  float* part;    // split-tail partial O and (m, l, xmax)
   float* stats;
-  unsigned int* count;  // [kFaCountWords] arrivals per (group, chain, quarter); units taken
+  unsigned int* count;  // units taken (split parts), zero at the start
   unsigned int* err;
   int parts_only;       // 1: the split-parts instance runs alone and takes every unit
 };
-
-// The work of one launch: G groups (head, kChains query tiles) over P persistent CTAs.  The
-// first R = floor(G / P) rounds take whole groups; the T = G - R P groups of the last round
-// are split along the keys into S parts each (at most the number of key tiles), T S part units,
-// so the last round lasts about ceil(T S / P) parts of a group instead of one whole group on T
-// CTAs.  Unit u < R P is group u; unit R P + S t + s is part s of group R P + t.
-// From kShortTiles key tiles on, S minimises the last round's length in key tiles,
-//   ceil(T S / P) (n_kv / S + kUnitTiles) + kCombineTiles S   (S = 1: no combine).
-// kUnitTiles, the cost of a unit beyond its keys (Q load, pipeline fill and drain, partial store
-// and arrival, about 10 us), and kCombineTiles, what a part adds to the combine (about 1 us), are
-// fitted to a sweep of S at 10,992 tokens; being costs in time they do not shrink with n_kv.
-// Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
-// 10,992 tokens 466 -> 394 us (8 groups left over: 19 parts -> 11), 3 heads 166 -> 122, 1 head at
-// 15,432 tokens 101 -> 92.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
-// 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
-// there: a deep stack of short sequences then gives the same bits as it always did.
-constexpr int kMaxParts = 64;
-constexpr int kMaxTailUnits = kFaTailUnits * 4 / kChains;  // the scratch is sized for four chains
-constexpr float kUnitTiles = 13.f, kCombineTiles = 1.5f;
-constexpr int kShortTiles = 41;
-constexpr float kPartShare = 0.03f;
-
-// Called by whole warps: lane l weighs S = l + 1 and l + 33 (a loop over S in every thread took
-// several microseconds of every launch).
-__device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_only) {
-  static_assert(kMaxParts == 64, "two values of S per lane");
-  Plan pl;
-  pl.R = G / P;
-  pl.T = G - pl.R * P;
-  pl.S = 1;
-  if (pl.T > 0) {
-    float best = INFINITY;
-    int bs = 1;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int S = lane_id() + 1 + 32 * k;
-      const bool brief = n_kv < kShortTiles;
-      if (S > 1 && (S > n_kv || pl.T * S > (brief ? kFaTailUnits : kMaxTailUnits))) continue;
-      const float rounds = (float)((pl.T * S + P - 1) / P);
-      const float cost = brief ? (S == 1 ? 1.f : rounds * (1.f / (float)S + kPartShare))
-                               : rounds * ((float)n_kv / (float)S + kUnitTiles) +
-                                     (S > 1 ? kCombineTiles * (float)S : 0.f);
-      if (cost < best) {
-        best = cost;
-        bs = S;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {  // smallest cost, then smallest S: the same on every lane
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int os = __shfl_xor_sync(0xffffffffu, bs, o);
-      if (ob < best || (ob == best && os < bs)) {
-        best = ob;
-        bs = os;
-      }
-    }
-    pl.S = bs;
-  }
-  pl.units = pl.S == 1 ? G : pl.R * P + pl.T * pl.S;
-  pl.whole = parts_only ? 0 : (pl.S == 1 ? G : pl.R * P);
-  return pl;
-}
 
 struct Unit {
   int group;       // head slot * n_groups + query-tile group
   int j0, nk;      // key tiles [j0, j0 + nk)
   int slot;        // split-tail slot (t S + s), -1 for a whole group
-  int tail;        // t
 };
 
 __device__ __forceinline__ Unit whole_unit(int u, int n_kv) {
@@ -182,7 +109,6 @@ __device__ __forceinline__ Unit whole_unit(int u, int n_kv) {
   w.j0 = 0;
   w.nk = n_kv;
   w.slot = -1;
-  w.tail = -1;
   return w;
 }
 
@@ -193,29 +119,23 @@ __device__ __forceinline__ Unit unit_of(const Plan& pl, int u, int P, int n_kv) 
     w.j0 = 0;
     w.nk = n_kv;
     w.slot = -1;
-    w.tail = -1;
-  } else {
+    } else {
     const int v = u - pl.R * P, t = v / pl.S, sp = v - t * pl.S;
     w.group = pl.R * P + t;
     w.j0 = sp * n_kv / pl.S;
     w.nk = (sp + 1) * n_kv / pl.S - w.j0;
     w.slot = v;
-    w.tail = t;
   }
   return w;
 }
 
 // Split-tail epilogue of one warp (32 rows of chain c, TMEM lanes at t_o): reads the part's
-// unnormalised O rows, releases O_c (o_empty), and publishes them with (m, l, xmax); the last
-// part of this (group, chain, lane quarter) to arrive combines all parts, M = max m_s,
-// O = sum 2^(m_s - M) O_s, l = sum 2^(m_s - M) l_s, and stores Y and the saliency.  A part's
-// 32 x 64 block lies lane-minor ([16-byte chunk][lane]), so that every store and load of a warp
-// is 512 contiguous bytes, and the combine works on half a row at a time with the loads of two
-// parts in flight.  Not inlined, and given only values: the attention loop's code and registers
-// stay as they are without it.
-__device__ __noinline__ void split_part(FullParams prm, int S, int part_slot, int tail, int c,
-                                        int quarter, int lane, int row, int h, uint32_t t_o,
-                                        uint64_t* o_empty, float m, float lsum, float xmax) {
+// unnormalised O rows, releases O_c (o_empty), and publishes them with (m, l, xmax) for
+// combine_split_heads (attn_plan.cuh).  Not inlined, and given only values: the attention loop's
+// code and registers stay as they are without it.
+__device__ __noinline__ void split_part(FullParams prm, int part_slot, int c, int quarter, int lane,
+                                        int row, int h, uint32_t t_o, uint64_t* o_empty, float m,
+                                        float lsum, float xmax) {
   float o[64];
   tmem_ld32(t_o, o);
   tmem_ld32(t_o + 32, o + 32);
@@ -244,76 +164,12 @@ __device__ __noinline__ void split_part(FullParams prm, int S, int part_slot, in
     }
     return;
   }
-  constexpr size_t kSlot = (size_t)kChains * 4 * 32;  // rows of a slot: [chain][quarter][lane]
-  const size_t blk = (size_t)(c * 4 + quarter) * 32;
-  float4* po = reinterpret_cast<float4*>(prm.part) + (part_slot * kSlot + blk) * 16 + lane;
+  const size_t blk = part_slot * kFaSlotRows + (size_t)(c * 4 + quarter) * 32;
+  float4* po = reinterpret_cast<float4*>(prm.part) + blk * 16 + lane;
 #pragma unroll
   for (int q = 0; q < 16; ++q)
     po[q * 32] = make_float4(o[4 * q], o[4 * q + 1], o[4 * q + 2], o[4 * q + 3]);
-  float4* stats = reinterpret_cast<float4*>(prm.stats) + blk + lane;
-  stats[part_slot * kSlot] = make_float4(m, lsum, xmax, 0.f);
-  __threadfence();
-  __syncwarp();
-  unsigned int last = 0;
-  if (lane == 0)
-    last = atomicAdd(prm.count + (tail * 4 + c) * 4 + quarter, 1u) == (unsigned)(S - 1);
-  if (!__shfl_sync(0xffffffffu, last, 0)) return;
-  __threadfence();
-  const size_t slot0 = (size_t)tail * S;
-  const float4* st = stats + slot0 * kSlot;
-  float M = -INFINITY, X = -INFINITY;
-#pragma unroll 8
-  for (int sp = 0; sp < S; ++sp) {
-    const float4 st4 = __ldcg(st + sp * kSlot);
-    M = fmaxf(M, st4.x);
-    X = fmaxf(X, st4.z);
-  }
-  float L = 0.f;
-#pragma unroll 8
-  for (int sp = 0; sp < S; ++sp) {
-    const float4 st4 = __ldcg(st + sp * kSlot);
-    L = fmaf(fast_exp2(st4.x - M), st4.y, L);
-  }
-  const float inv = 1.f / L;
-#pragma unroll 1
-  for (int half = 0; half < 2; ++half) {
-    const float4* pq = reinterpret_cast<const float4*>(prm.part) + (slot0 * kSlot + blk) * 16 + lane + half * 256;
-    float acc[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) acc[i] = 0.f;
-#pragma unroll 2
-    for (int sp = 0; sp < S; ++sp) {
-      const float wgt = fast_exp2(__ldcg(&st[sp * kSlot].x) - M);
-      float4 f[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) f[q] = __ldcg(pq + sp * kSlot * 16 + q * 32);
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        acc[4 * q] = fmaf(wgt, f[q].x, acc[4 * q]);
-        acc[4 * q + 1] = fmaf(wgt, f[q].y, acc[4 * q + 1]);
-        acc[4 * q + 2] = fmaf(wgt, f[q].z, acc[4 * q + 2]);
-        acc[4 * q + 3] = fmaf(wgt, f[q].w, acc[4 * q + 3]);
-      }
-    }
-    if (row < prm.N) {
-      uint4* dst = reinterpret_cast<uint4*>(prm.y + ((size_t)row * prm.H + h) * 64) + half * 4;
-#pragma unroll
-      for (int ch = 0; ch < 4; ++ch) {
-        uint4 v;
-        v.x = pack_bf16x2(acc[8 * ch + 0] * inv, acc[8 * ch + 1] * inv);
-        v.y = pack_bf16x2(acc[8 * ch + 2] * inv, acc[8 * ch + 3] * inv);
-        v.z = pack_bf16x2(acc[8 * ch + 4] * inv, acc[8 * ch + 5] * inv);
-        v.w = pack_bf16x2(acc[8 * ch + 6] * inv, acc[8 * ch + 7] * inv);
-        dst[ch] = v;
-      }
-    }
-  }
-  if (prm.s_attn) {
-    float a = row < prm.N ? fast_exp2(X - M) * inv : 0.f;
-#pragma unroll
-    for (int k = 16; k > 0; k >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, k));
-    if (lane == 0) atomicMax(reinterpret_cast<int*>(prm.s_attn + h), __float_as_int(a));
-  }
+  reinterpret_cast<float4*>(prm.stats)[blk + lane] = make_float4(m, lsum, xmax, 0.f);
 }
 
 // kParts = false: the whole groups (all of them when nothing is split); kParts = true: the
@@ -424,7 +280,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive(&sm.unit_full[ic % kUnitSlots]);
         }
         __syncwarp();
-        if (lane == 0) taken = (int)atomicAdd(prm.count + kFaUnitCounter, 1u);
+        if (lane == 0) taken = (int)atomicAdd(prm.count, 1u);
         __syncwarp();
       }
       const Unit w = kParts ? unit_of(plan, u, P, n_kv) : whole_unit(u, n_kv);
@@ -686,8 +542,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_after();
       const int row = (qg * kChains + c) * kBM + row_in_tile;
       if (kParts) {  // a part of a split group (the last round's groups), or a whole group
-        split_part(prm, plan.S, w.slot, w.tail, c, quarter, lane, row, h, t_o, &sm.o_empty[c], m, lsum,
-                   xmax);
+        split_part(prm, w.slot, c, quarter, lane, row, h, t_o, &sm.o_empty[c], m, lsum, xmax);
         __syncwarp();
         continue;
       }
@@ -753,7 +608,7 @@ cudaError_t launch_full_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t s
   const int groups_max = a.H * ((a.N + kChains * kBM - 1) / (kChains * kBM));
   const bool parts_only = groups_max <= num_sms;
   FullParams prm{a.N, a.H, a.head_ids, a.offsets, a.y, a.s_attn, a.fa_part, a.fa_stats,
-                 a.fa_count, a.err, parts_only ? 1 : 0};
+                 a.counters + kFaUnitCounter, a.err, parts_only ? 1 : 0};
   if (!parts_only) {
     e = launch_pdl(attn_full_kernel<false>, dim3(num_sms), kThreads, smem, st, tmap_q, tmap_kv, prm);
     if (e != cudaSuccess) return e;

@@ -1,0 +1,160 @@
+// How the full-attention work of a layer is cut (attn_full.cu), and the combine of the groups that
+// were split along the keys, which the kernel behind the attention runs (combine_split_heads).
+#pragma once
+
+#include <math.h>
+
+#include "common.cuh"
+#include "internal.h"
+
+namespace vp {
+
+#ifndef VP_ATTN_CHAINS
+#define VP_ATTN_CHAINS 3
+#endif
+#ifndef VP_ATTN_BN
+#define VP_ATTN_BN 64
+#endif
+constexpr int kFaChains = VP_ATTN_CHAINS;  // query tiles (chains) of a group
+constexpr int kFaRows = 128;               // query rows of a tile
+constexpr int kFaKeys = VP_ATTN_BN;        // keys of a tile
+
+struct Plan {
+  int R, T, S, units;
+  int whole;  // units of the whole-group instance (they come first)
+};
+
+// The work of one launch: G groups (head, kFaChains query tiles) over P persistent CTAs.  The
+// first R = floor(G / P) rounds take whole groups; the T = G - R P groups of the last round
+// are split along the keys into S parts each (at most the number of key tiles), T S part units,
+// so the last round lasts about ceil(T S / P) parts of a group instead of one whole group on T
+// CTAs.  Unit u < R P is group u; unit R P + S t + s is part s of group R P + t.
+// From kShortTiles key tiles on, S minimises the last round's length in key tiles,
+//   ceil(T S / P) (n_kv / S + kUnitTiles) + kCombineTiles S   (S = 1: no combine).
+// kUnitTiles, the cost of a unit beyond its keys (Q load, pipeline fill and drain, partial store),
+// and kCombineTiles, what a part adds to the combine, are fitted to a sweep of S at 10,992
+// tokens; being costs in time they do not shrink with n_kv.
+// Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
+// 10,992 tokens 466 -> 394 us (8 groups left over: 19 parts -> 11), 3 heads 166 -> 119, 1 head at
+// 15,432 tokens 101 -> 92.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
+// 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
+// there: a deep stack of short sequences then gives the same bits as it always did.
+constexpr int kMaxParts = 64;
+constexpr int kMaxTailUnits = kFaTailUnits * 4 / kFaChains;  // the scratch is sized for four chains
+constexpr float kUnitTiles = 13.f, kCombineTiles = 1.5f;
+constexpr int kShortTiles = 41;
+constexpr float kPartShare = 0.03f;
+
+// Called by whole warps: lane l weighs S = l + 1 and l + 33 (a loop over S in every thread took
+// several microseconds of every launch).
+__device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_only) {
+  static_assert(kMaxParts == 64, "two values of S per lane");
+  Plan pl;
+  pl.R = G / P;
+  pl.T = G - pl.R * P;
+  pl.S = 1;
+  if (pl.T > 0) {
+    float best = INFINITY;
+    int bs = 1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int S = lane_id() + 1 + 32 * k;
+      const bool brief = n_kv < kShortTiles;
+      if (S > 1 && (S > n_kv || pl.T * S > (brief ? kFaTailUnits : kMaxTailUnits))) continue;
+      const float rounds = (float)((pl.T * S + P - 1) / P);
+      const float cost = brief ? (S == 1 ? 1.f : rounds * (1.f / (float)S + kPartShare))
+                               : rounds * ((float)n_kv / (float)S + kUnitTiles) +
+                                     (S > 1 ? kCombineTiles * (float)S : 0.f);
+      if (cost < best) {
+        best = cost;
+        bs = S;
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {  // smallest cost, then smallest S: the same on every lane
+      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
+      const int os = __shfl_xor_sync(0xffffffffu, bs, o);
+      if (ob < best || (ob == best && os < bs)) {
+        best = ob;
+        bs = os;
+      }
+    }
+    pl.S = bs;
+  }
+  pl.units = pl.S == 1 ? G : pl.R * P + pl.T * pl.S;
+  pl.whole = parts_only ? 0 : (pl.S == 1 ? G : pl.R * P);
+  return pl;
+}
+
+// A part's rows in the scratch: slot t S + s holds [chain][quarter] blocks of 32 rows (lanes); a
+// block's O lies lane-minor ([16-byte chunk of the row][lane]), its (m, l, xmax) a float4 per lane,
+// so that every store and load of a warp is 512 contiguous bytes.
+constexpr size_t kFaSlotRows = (size_t)kFaChains * 4 * 32;
+
+// The split groups' rows of Y (and their share of the saliency) from the parts of a finished
+// attention launch over P CTAs: M = max m_s, O = sum 2^(m_s - M) O_s, l = sum 2^(m_s - M) l_s,
+// parts in order.  Called by whole warps, warp w of n_warps of the grid behind the attention
+// kernel: a warp takes 8 channels of a block of 32 rows at a time, so the partial rows come in
+// over every SM (one group's are up to 1.7 MB; the last part's CTA on its own took 15 us for
+// them at 1,044 tokens).
+// Not inlined: the kernels that end with it keep their code and registers.
+static __device__ __noinline__ void combine_split_heads(const HeadAttnArgs& a, int P, int w, int n_warps) {
+  const int first = a.offsets[2], n_heads = a.offsets[3] - first;
+  const int n_groups = (a.N + kFaChains * kFaRows - 1) / (kFaChains * kFaRows);
+  const Plan pl = make_plan(n_heads * n_groups, P, (a.N + kFaKeys - 1) / kFaKeys, false);
+  if (pl.S == 1) return;
+  const int lane = lane_id();
+  for (int task = w; task < pl.T * kFaChains * 32; task += n_warps) {
+    const int piece = task & 7, quarter = (task >> 3) & 3, ct = task >> 5;
+    const int t = ct / kFaChains, c = ct - t * kFaChains;
+    const int group = pl.R * P + t;
+    const int h = a.head_ids[first + group / n_groups];
+    const int row = ((group % n_groups) * kFaChains + c) * kFaRows + quarter * 32 + lane;
+    const size_t blk = (size_t)t * pl.S * kFaSlotRows + (size_t)(c * 4 + quarter) * 32;
+    const float4* st = reinterpret_cast<const float4*>(a.fa_stats) + blk + lane;
+    const float4* pq = reinterpret_cast<const float4*>(a.fa_part) + blk * 16 + piece * 64 + lane;
+    float M = -INFINITY, X = -INFINITY;
+#pragma unroll 8
+    for (int sp = 0; sp < pl.S; ++sp) {
+      const float4 s4 = __ldcg(st + sp * kFaSlotRows);
+      M = fmaxf(M, s4.x);
+      X = fmaxf(X, s4.z);
+    }
+    float L = 0.f, acc[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) acc[i] = 0.f;
+#pragma unroll 6
+    for (int sp = 0; sp < pl.S; ++sp) {
+      const float2 s4 = __ldcg(reinterpret_cast<const float2*>(st + sp * kFaSlotRows));
+      float4 f[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) f[q] = __ldcg(pq + sp * kFaSlotRows * 16 + q * 32);
+      const float wgt = fast_exp2(s4.x - M);
+      L = fmaf(wgt, s4.y, L);
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        acc[4 * q] = fmaf(wgt, f[q].x, acc[4 * q]);
+        acc[4 * q + 1] = fmaf(wgt, f[q].y, acc[4 * q + 1]);
+        acc[4 * q + 2] = fmaf(wgt, f[q].z, acc[4 * q + 2]);
+        acc[4 * q + 3] = fmaf(wgt, f[q].w, acc[4 * q + 3]);
+      }
+    }
+    const float inv = 1.f / L;
+    if (row < a.N) {
+      uint4 v;
+      v.x = pack_bf16x2(acc[0] * inv, acc[1] * inv);
+      v.y = pack_bf16x2(acc[2] * inv, acc[3] * inv);
+      v.z = pack_bf16x2(acc[4] * inv, acc[5] * inv);
+      v.w = pack_bf16x2(acc[6] * inv, acc[7] * inv);
+      reinterpret_cast<uint4*>(a.y + ((size_t)row * a.H + h) * 64)[piece] = v;
+    }
+    if (a.s_attn && piece == 0) {
+      float v = row < a.N ? fast_exp2(X - M) * inv : 0.f;
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, k));
+      if (lane == 0) atomicMax(reinterpret_cast<int*>(a.s_attn + h), __float_as_int(v));
+    }
+  }
+}
+
+}  // namespace vp

@@ -434,7 +434,7 @@ __device__ __forceinline__ float bf16_hi(uint32_t u) { return __uint_as_float(u 
 
 // Column n of W_O's bias with the mean heads folded in (internal.h, launch_wo_mean_fold), by one
 // warp: lane l takes channels 2 l, 2 l + 1 of the mean heads head_ids[m0 .. m1).
-__device__ __forceinline__ void wo_mean_fold_column(int n, int H, const __nv_bfloat16* w_o,
+static __device__ __noinline__ void wo_mean_fold_column(int n, int H, const __nv_bfloat16* w_o,
                                                     const float* b_o, const float* mean_v,
                                                     const int32_t* head_ids, int m0, int m1,
                                                     float* bias_out) {

@@ -3,15 +3,16 @@
 // programmatic dependent launch (heads_cheap_tc.cu).  The full-attention CTAs signal their
 // dependents as soon as they start, so cheap-head CTAs take each SM as soon as a
 // full-attention CTA retires.  The cheap kernels read only router outputs (bins, C_h, mean of
-// V), which were complete before the full-attention kernel started; they wait for the
-// full-attention grid (griddepcontrol.wait) before they exit, so work queued after them sees
-// every head's Y.
+// V), which were complete before the full-attention kernel started; at their end they wait for
+// the full-attention grid (griddepcontrol.wait) and combine the groups it split along the keys
+// (combine_split_heads), so work queued after them sees every head's Y.
 //
 // Two §5 ablations change the cheap heads.  Linear attention replaces the surrogate: its two
 // tcgen05 kernels (linear_attn_tc.cu) run before the full-attention kernel.  Without the
 // token-wise correction a surrogate head is y_i = C_h, a broadcast like a mean head.  In both
 // variants broadcast_heads_kernel writes the broadcast rows (the no-residual surrogate heads and
 // the mean heads) behind the full-attention kernel.
+#include "attn_plan.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -67,8 +68,9 @@ __global__ void __launch_bounds__(kThreads, 3) broadcast_heads_kernel(HeadAttnAr
       broadcast_rows(a, a.mean_v + h * 64, h, chunk * kRows, tid);
     }
   }
-  // Do not complete before the full-attention grid: later work in the stream reads all of Y.
+  // Once the full-attention grid has completed: its split groups.
   pdl_wait();
+  combine_split_heads(a, a.attn_ctas, (tid >> 5) * (int)gridDim.x + (int)blockIdx.x, (kThreads / 32) * (int)gridDim.x);
 }
 
 }  // namespace
@@ -76,7 +78,7 @@ __global__ void __launch_bounds__(kThreads, 3) broadcast_heads_kernel(HeadAttnAr
 cudaError_t launch_heads(const HeadAttnArgs& a, int num_sms, cudaStream_t st) {
   cudaError_t e = cudaSuccess;
   if (!a.counters_zeroed) {
-    e = cudaMemsetAsync(a.fa_count, 0, sizeof(unsigned int) * kFaCountWords, st);
+    e = cudaMemsetAsync(a.counters, 0, sizeof(unsigned int) * kHeadCounters, st);
     if (e != cudaSuccess) return e;
     if (a.s_attn) {  // 0 for the heads that are not in full mode; full heads max into it
       e = cudaMemsetAsync(a.s_attn, 0, sizeof(float) * a.H, st);

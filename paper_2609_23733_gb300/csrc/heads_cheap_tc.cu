@@ -19,8 +19,6 @@
 //
 // Roles (576 threads, one CTA per SM, persistent over items taken kBatch at a time from a
 // device counter: surrogate tiles of 128 tokens head-major, then mean items of 1,024 tokens):
-//   all        at the start, every surrogate head's per-head vectors into shared memory
-//              (c1 = W1[:, d:] C_h + b1, the second layer's biases, C_h);
 //   warp 0     producer: items, TMA loads of the V tiles (kStages ring) and of each head's
 //              weights into one of two weight slots (a slot is reloaded once the MMAs of the
 //              head before the previous one have completed);
@@ -30,7 +28,9 @@
 //              g takes tiles t = g (mod 2).  Its j-th tile keeps D1, then D2g | D2d, in the
 //              128-column half j & 1 and H in the first 64 columns of the other half, so the
 //              first layer of its next tile (the other half) runs while it reads D2.  The
-//              two warps of a TMEM lane quarter split a token row's columns (kTcParts).
+//              two warps of a TMEM lane quarter split a token row's columns (kTcParts).  At the
+//              start they put the surrogate heads' vectors into shared memory (c1 = W1[:, d:] C_h
+//              + b1, the second layer's biases, C_h), beside the first copies and MMAs.
 // The register file is split between the four SM sub-partitions: 18 warps put 5 on some of
 // them, which caps a thread at 96 registers (16,384 / (5 x 32), in steps of 8).  Three warps
 // per lane quarter (26 warps, 72 registers) measured slower: 0.301 vs 0.269 ms for 16 heads
@@ -38,6 +38,7 @@
 // Every wait is bounded (mbar_wait); on timeout the CTA records VP_DEVERR_WAIT_TIMEOUT, stops,
 // waits (bounded) for its own copies and MMAs, frees TMEM and exits.  The groups agree on
 // stopping through reduction barriers, so that no thread is left at a named barrier.
+#include "attn_plan.cuh"
 #include "common.cuh"
 #include "internal.h"
 
@@ -49,7 +50,7 @@ constexpr int kTcTile = 128;      // tokens per surrogate item
 constexpr int kMeanRows = 1024;   // tokens per mean item (a pure write, handed over less often)
 constexpr int kTcStages = 4;      // V tiles in flight
 constexpr int kTcGroups = 2;      // epilogue groups (= TMEM accumulators)
-constexpr int kTcBatch = 4;       // items taken from the counter at a time
+constexpr int kTcBatch = 4;       // items taken from the counter at a time (one when there are few)
 constexpr int kTcParts = 2;       // epilogue warps per TMEM lane quarter in a group
 constexpr int kGroupThreads = 128 * kTcParts;
 constexpr int kTcThreads = 64 + kGroupThreads * kTcGroups;
@@ -85,6 +86,7 @@ struct TcSmem {
   uint64_t drain;
   uint32_t tmem_base;
   int abort_flag;
+  int first_item;  // the first batch's start
 };
 
 // Barrier over the threads of an epilogue group (named barrier 1 + g) that also returns
@@ -100,6 +102,32 @@ __device__ __forceinline__ bool group_all(bool p, int g) {
       : "r"((uint32_t)p), "r"(1 + g), "n"(kGroupThreads)
       : "memory");
   return r != 0;
+}
+
+// The vectors of the surrogate head h in slot: the first layer's context half folded into c1 (one
+// 64-term dot product per hidden unit), the second layer's biases, C_h; by the kGroupThreads
+// threads of a group.
+__device__ __noinline__ void head_vectors(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int gt) {
+  const int u = gt & 127, uu = u & 63;
+  if (gt < 128) {
+    const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
+    const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
+    float acc = (u < 64 ? a.sw.g1_b : a.sw.d1_b)[h * 64 + uu];
+#pragma unroll
+    for (int kq = 0; kq < 8; ++kq) {
+      const uint4 wv = reinterpret_cast<const uint4*>(w)[kq];
+      const float4 c0 = ctx[2 * kq], c1 = ctx[2 * kq + 1];
+      acc = fmaf(bf16_lo(wv.x), c0.x, fmaf(bf16_hi(wv.x), c0.y, acc));
+      acc = fmaf(bf16_lo(wv.y), c0.z, fmaf(bf16_hi(wv.y), c0.w, acc));
+      acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
+      acc = fmaf(bf16_lo(wv.w), c1.z, fmaf(bf16_hi(wv.w), c1.w, acc));
+    }
+    sm.c1[slot][u] = acc;
+  } else {
+    const float b = (u < 64 ? a.sw.g2_b : a.sw.d2_b)[h * 64 + uu];
+    sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
+    if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
+  }
 }
 
 struct TcMaps {
@@ -122,9 +150,13 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
   const int Tm = (a.N + kMeanRows - 1) / kMeanRows;  // mean items per head
   // Mean heads folded into W_O's bias (skip_mean_y) need no rows of Y.
   const int items = surr_items + (a.skip_mean_y ? 0 : n_mean * Tm);
+  // With fewer than two batches per CTA, items go out one by one (63 items of one 1,044-token layer:
+  // 16 CTAs took four each, one after another).
+  const int batch = items > 2 * kTcBatch * (int)gridDim.x ? kTcBatch : 1;
 
   pdl_launch();
   if (tid == 0) {
+    sm.first_item = (int)atomicAdd(a.cheap_counter, (unsigned)batch);
     for (int s = 0; s < kTcStages; ++s) {
       mbar_init(&sm.full[s], 1);
       mbar_init(&sm.empty[s], 1);
@@ -150,42 +182,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     tmem_alloc(&sm.tmem_base, kTcTmemCols);
     tmem_relinquish();
   }
-  // The mean heads folded into W_O's bias (launch_wo_mean_fold's arithmetic), a warp per output
-  // column: a launch of its own between the router and the heads cost 4-5 us a layer.
-  if (a.wo_bias) {
-    for (int n = (int)blockIdx.x * (kTcThreads / 32) + warp; n < H * 64; n += (int)gridDim.x * (kTcThreads / 32))
-      wo_mean_fold_column(n, H, a.w_o, a.b_o, a.mean_v, a.head_ids, m_first, s_first, a.wo_bias);
-  }
-  // The surrogate heads' per-head vectors: the first layer's context half folded into c1 (one
-  // 64-term dot product per hidden unit), the second layer's biases, C_h.
-  for (int i = tid; i < n_surr * 128; i += kTcThreads) {
-    const int slot = i >> 7, u = i & 127, uu = u & 63;
-    const int h = a.head_ids[s_first + slot];
-    const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
-    const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
-    float acc = __ldg((u < 64 ? a.sw.g1_b : a.sw.d1_b) + h * 64 + uu);
-#pragma unroll
-    for (int kq = 0; kq < 8; ++kq) {
-      const uint4 wv = __ldg(reinterpret_cast<const uint4*>(w) + kq);
-      const float4 c0 = ctx[2 * kq], c1 = ctx[2 * kq + 1];
-      acc = fmaf(bf16_lo(wv.x), c0.x, fmaf(bf16_hi(wv.x), c0.y, acc));
-      acc = fmaf(bf16_lo(wv.y), c0.z, fmaf(bf16_hi(wv.y), c0.w, acc));
-      acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
-      acc = fmaf(bf16_lo(wv.w), c1.z, fmaf(bf16_hi(wv.w), c1.w, acc));
-    }
-    sm.c1[slot][u] = acc;
-    const float b = __ldg((u < 64 ? a.sw.g2_b : a.sw.d2_b) + h * 64 + uu);
-    sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
-    if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
 
-  if (warp == 0) {
+  // A CTA that starts behind the attention's last round may find every item taken: it goes
+  // straight to the combine.
+  const int first_item = __shfl_sync(0xffffffffu, sm.first_item, 0);
+  if (first_item >= items) {
+  } else if (warp == 0) {
     // ------------------------------------------------------------ producer
-    int fill = -1, cur_h = -1, next = 0, left = 0;
+    int fill = -1, cur_h = -1, next = first_item, left = batch;
     int tma_k[kTcStages];  // last item index k whose V tile went to stage s (-1: none)
 #pragma unroll
     for (int s = 0; s < kTcStages; ++s) tma_k[s] = -1;
@@ -193,9 +201,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     for (int k = 0;; ++k) {
       if (left == 0) {
         int b = 0;
-        if (lane == 0) b = (int)atomicAdd(a.cheap_counter, (unsigned)kTcBatch);
+        if (lane == 0) b = (int)atomicAdd(a.cheap_counter, (unsigned)batch);
         next = __shfl_sync(0xffffffffu, b, 0);
-        left = kTcBatch;
+        left = batch;
       }
       const int it = next++;
       --left;
@@ -456,6 +464,19 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     const int f0 = part_begin(kTcParts - 1 - part, 4), f1 = part_begin(kTcParts - part, 4);
     uint32_t sj = 0;  // surrogate tiles of this group
     bool ok = true;
+    // The heads' vectors: all of them now, while the first tile's copies and MMAs run, or with
+    // single items (few of a CTA's heads are ever used) each when a tile first needs it.
+    uint32_t ready = 0;  // heads (by slot) whose vectors this group has seen to
+    if (batch > 1) {
+      for (int sl = 0; sl < n_surr; sl += 2)
+        if (sl + g < n_surr) head_vectors(a, sm, sl + g, a.head_ids[s_first + sl + g], gt);
+      ready = 0xffffffffu;
+      asm volatile("bar.sync 3, %0;" ::"n"(kGroupThreads * kTcGroups) : "memory");
+    } else if (g == 0 && first_item < surr_items) {
+      const int sl = first_item / T;
+      head_vectors(a, sm, sl, a.head_ids[s_first + sl], gt);
+      ready = 1u << sl;  // seen by the group behind the barrier below
+    }
     for (uint32_t j = 0;; ++j) {
       ok = group_all(mbar_wait_warp(&sm.d1_full[g], j & 1, err, abort_flag), g);
       if (!ok) break;
@@ -466,6 +487,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
       const bool surr = it < surr_items;
       const int tile = surr ? it % T : (it - surr_items) % Tm;  // a mean item spans kMeanRows rows
       const int slot = surr ? it / T : 0;  // surrogate head slot: its vectors
+      if (surr && !((ready >> slot) & 1u)) {
+        head_vectors(a, sm, slot, h, gt);
+        ready |= 1u << slot;
+        group_all(true, g);
+      }
       const float* c1 = sm.c1[slot];
       const float* b2 = sm.b2[slot];
       const float* cx = sm.cx[slot];
@@ -578,8 +604,23 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     tc_fence_after();
     tmem_dealloc(tmem, kTcTmemCols);
   }
-  // Do not complete before the full-attention grid: later work in the stream reads all of Y.
-  if (tid == 0) pdl_wait();
+  // The mean heads folded into W_O's bias, a warp per output column (a launch of its own between
+  // the router and the heads cost 4-5 us a layer); the columns from a counter, so that the CTAs
+  // without items take them.
+  if (a.wo_bias) {
+    for (;;) {
+      if (tid == 0) sm.first_item = (int)atomicAdd(a.fold_counter, (unsigned)(kTcThreads / 32));
+      __syncthreads();
+      const int n0 = sm.first_item;
+      __syncthreads();
+      if (n0 >= H * 64) break;
+      if (n0 + warp < H * 64)
+        wo_mean_fold_column(n0 + warp, H, a.w_o, a.b_o, a.mean_v, a.head_ids, m_first, s_first, a.wo_bias);
+    }
+  }
+  // Once the full-attention grid has completed: its split groups, spread over all warps.
+  pdl_wait();
+  combine_split_heads(a, a.attn_ctas, warp * (int)gridDim.x + (int)blockIdx.x, (kTcThreads / 32) * (int)gridDim.x);
 }
 
 }  // namespace

@@ -39,7 +39,7 @@ struct RouterScratch {
   float* lin_state;             // [H][kLinState] linear-attention state (after the router part)
   float* fa_part;               // split-tail partial O, kFaPartFloats (layout: attn_full.cu)
   float* fa_stats;              // its (m, l, xmax, -) rows, kFaStatsFloats
-  unsigned int* fa_count;       // kFaCountWords: split arrivals, then the counters named below
+  unsigned int* head_counters;  // [kHeadCounters] counters of the head modes, zeroed per call
   float* wo_bias;               // [kMaxHeads * 64] W_O bias with the mean heads folded in
 };
 
@@ -49,9 +49,8 @@ struct RouterScratch {
 constexpr int kFaTailUnits = 512;
 constexpr size_t kFaPartFloats = (size_t)kFaTailUnits * 4 * 128 * 64;
 constexpr size_t kFaStatsFloats = (size_t)kFaTailUnits * 4 * 128 * 4;
-constexpr size_t kFaCountWords = (size_t)kFaTailUnits * 4 * 4;
-// The last words of that scratch count the split parts and the cheap-head items handed out.
-constexpr size_t kFaUnitCounter = kFaCountWords - 1, kCheapCounter = kFaCountWords - 2;
+// Counters of the head modes: split parts, cheap-head items and columns of W_O's bias handed out.
+constexpr int kHeadCounters = 64, kFaUnitCounter = 0, kCheapCounter = 32, kFoldCounter = 33;
 
 // Linear-attention state of one head (the §5 compute-mode ablation): S_h [64 c][64 e] =
 // sum_j phi(k_j)[c] v_j[e], then z_h [64] = sum_j phi(k_j), fp32.
@@ -86,9 +85,8 @@ struct RouterArgs {
   const float* beta;
   const int32_t* force_modes;
   // Counters of the head modes that the router clears on its way (a layer's heads run behind it):
-  // zero_words words from zero, and s_attn_zero [H]; NULL: none.
-  unsigned int* zero;
-  int zero_words;
+  // head_counters [kHeadCounters] and s_attn_zero [H]; NULL: none.
+  unsigned int* head_counters;
   float* s_attn_zero;
   // Outputs (NULL = do not copy out); the scratch copies are always written.
   float* s_out;
@@ -133,16 +131,18 @@ struct HeadAttnArgs {
   float* lin_state;             // [H][kLinState] (VP_VARIANT_LINEAR_ATTENTION only)
   float* fa_part;               // split-tail scratch of the full-attention kernel
   float* fa_stats;
-  unsigned int* fa_count;       // zeroed by launch_heads, or before it (counters_zeroed)
+  unsigned int* counters;       // [kHeadCounters], zeroed by launch_heads or before it (counters_zeroed)
+  int attn_ctas;                // grid of the full-attention kernel
   unsigned int* err;
-  unsigned int* cheap_counter;  // fa_count[kCheapCounter]
-  int counters_zeroed;          // 1: fa_count and s_attn were cleared earlier in the stream
+  unsigned int* cheap_counter;  // counters[kCheapCounter]
+  int counters_zeroed;          // 1: counters and s_attn were cleared earlier in the stream
   int skip_mean_y;              // 1: the mean heads' rows of Y are not written (folded into W_O)
   // The mean heads folded into W_O's bias by the cheap-heads kernel (see launch_wo_mean_fold):
   // wo_bias[n], n < 64 H, from W_O and b_O (NULL: 0); wo_bias NULL: not here.
   const __nv_bfloat16* w_o;
   const float* b_o;
   float* wo_bias;
+  unsigned int* fold_counter;   // counters[kFoldCounter]
 };
 
 // Full-mode heads (attn_full.cu).

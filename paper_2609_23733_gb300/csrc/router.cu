@@ -139,11 +139,11 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
   pdl_wait();
   pdl_launch();
   {  // counters of the key sweep, and of the head modes where they follow
-    const int cta = blockIdx.y * gridDim.x + blockIdx.x, step = gridDim.x * gridDim.y * kPoolTcThreads;
-    if (cta == 0 && tid < 128) sc.counters[tid] = 0u;
-    if (a.zero)
-      for (int i = cta * kPoolTcThreads + tid; i < a.zero_words; i += step) a.zero[i] = 0u;
-    if (a.s_attn_zero && cta == 0 && tid < a.H) a.s_attn_zero[tid] = 0.f;
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+      if (tid < 128) sc.counters[tid] = 0u;
+      if (a.head_counters && tid < kHeadCounters) a.head_counters[tid] = 0u;
+      if (a.s_attn_zero && tid < a.H) a.s_attn_zero[tid] = 0.f;
+    }
   }
   if (tid < 64) {
     sm.bias[tid] = a.bW ? a.bW[h * 64 + tid] : 0.f;
@@ -642,7 +642,7 @@ cudaError_t launch_wait_selftest(unsigned int* err, unsigned long long limit_ns,
 
 size_t heads_scratch_bytes(int H) {
   return router_scratch_bytes(H) + (size_t)kMaxHeads * kLinState * 4 +
-         (kFaPartFloats + kFaStatsFloats + kFaCountWords) * 4 + (size_t)kMaxHeads * 64 * 4;
+         (kFaPartFloats + kFaStatsFloats + kHeadCounters) * 4 + (size_t)kMaxHeads * 64 * 4;
 }
 
 RouterScratch carve_router_scratch(void* ws, int H) {
@@ -674,8 +674,8 @@ RouterScratch carve_router_scratch(void* ws, int H) {
   sc.lin_state = reinterpret_cast<float*>(static_cast<char*>(ws) + router_scratch_bytes(H));
   sc.fa_part = sc.lin_state + (size_t)kMaxHeads * kLinState;
   sc.fa_stats = sc.fa_part + kFaPartFloats;
-  sc.fa_count = reinterpret_cast<unsigned int*>(sc.fa_stats + kFaStatsFloats);
-  sc.wo_bias = reinterpret_cast<float*>(sc.fa_count + kFaCountWords);
+  sc.head_counters = reinterpret_cast<unsigned int*>(sc.fa_stats + kFaStatsFloats);
+  sc.wo_bias = reinterpret_cast<float*>(sc.head_counters + kHeadCounters);
   return sc;
 }
 
