@@ -24,20 +24,25 @@
 //              head before the previous one have completed);
 //   warp 1     TMEM owner (512 columns) and MMA issue: the first layer of the next tile and
 //              the second layer of a tile whose H is written, each as soon as it is ready;
-//   warps 2-9, 10-17  two epilogue groups of eight warps, each with 256 TMEM columns; group
-//              g takes tiles t = g (mod 2).  Its j-th tile keeps D1, then D2g | D2d, in the
-//              128-column half j & 1 and H in the first 64 columns of the other half, so the
-//              first layer of its next tile (the other half) runs while it reads D2.  The
-//              two warps of a TMEM lane quarter split a token row's columns (kTcParts).  At the
-//              start they put the surrogate heads' vectors into shared memory (c1 = W1[:, d:] C_h
-//              + b1, the second layer's biases, C_h), beside the first copies and MMAs.
+//   warps 2-9, 10-17  two epilogue groups of eight warps, each with 256 TMEM columns; group g takes
+//              tiles t = g (mod 2): D1 and, in place, H in its first 128 columns, D2g | D2d in
+//              the other 128.  The tensor pipe runs the MMAs in the order of issue, so the first
+//              layer of the group's next tile goes out right behind the second layer that reads
+//              H.  The two warps of a TMEM lane quarter split a token row's columns, and no warp
+//              waits for another one: each stages and stores its own 32 x 32 block of y (TMA),
+//              and the hand-overs are mbarriers.  With group barriers around a staged tile (three
+//              a tile) the same work took 171 us for 16 surrogate heads at 87,936 tokens, now 165.
+//              The surrogate heads' vectors (c1 = W1[:, d:] C_h + b1, the second layer's biases,
+//              C_h) are put into shared memory beside the first copies and MMAs.
+// Bounded by the latency of that chain with two tiles in flight: issue, FMA and MUFU are each below
+// half of their rate.  All 16 warps on one tile at a time, the gate one tile behind, measured slower
+// (184 vs 171 us): the phases of the warps then coincide.
 // The register file is split between the four SM sub-partitions: 18 warps put 5 on some of
 // them, which caps a thread at 96 registers (16,384 / (5 x 32), in steps of 8).  Three warps
 // per lane quarter (26 warps, 72 registers) measured slower: 0.301 vs 0.269 ms for 16 heads
 // at 137,400 tokens.
 // Every wait is bounded (mbar_wait); on timeout the CTA records VP_DEVERR_WAIT_TIMEOUT, stops,
-// waits (bounded) for its own copies and MMAs, frees TMEM and exits.  The groups agree on
-// stopping through reduction barriers, so that no thread is left at a named barrier.
+// waits (bounded) for its own copies and MMAs, frees TMEM and exits.
 #include "attn_plan.cuh"
 #include "common.cuh"
 #include "internal.h"
@@ -70,7 +75,7 @@ struct TcSmem {
   __nv_bfloat16 v[kTcStages][kTcTile * 64];
   __nv_bfloat16 w1[2][128 * 64];
   __nv_bfloat16 w2[2][128 * 64];
-  __nv_bfloat16 ys[kTcGroups][kTcTile * 64];  // output staging, 128-byte swizzle
+  __nv_bfloat16 ys[4 * kTcParts * kTcGroups][32 * 32];  // a warp's output block, 64-byte swizzle
   // Every surrogate head's vectors, by slot in the surrogate bin, computed at kernel start:
   // W1[:, d:] C_h + b1 (gamma | delta), -log2(e) b2_gamma | b2_delta, and C_h.
   float c1[kMaxHeads][128];
@@ -79,55 +84,39 @@ struct TcSmem {
   int stage_item[kTcStages];                  // item, or -1: no more items
   int stage_fill[kTcStages];                  // weight fill of a surrogate item (slot = fill & 1), -1
   int stage_head[kTcStages];
-  int acc_item[kTcGroups], acc_head[kTcGroups];
+  int stage_slot[kTcStages], stage_tile[kTcStages];  // item = slot x tiles + tile (divided once, here)
+  int acc_item[kTcGroups], acc_head[kTcGroups], acc_slot[kTcGroups], acc_tile[kTcGroups];
   uint64_t full[kTcStages], empty[kTcStages];
   uint64_t w_full[2], w_empty[2];
-  uint64_t d1_full[kTcGroups], h_full[kTcGroups], d2_full[kTcGroups], taken[kTcGroups];
+  uint64_t d1_full[kTcGroups], h_full[kTcGroups], d2_full[kTcGroups], taken[kTcGroups], vec_full[kTcGroups];
   uint64_t drain;
   uint32_t tmem_base;
   int abort_flag;
   int first_item;  // the first batch's start
 };
 
-// Barrier over the threads of an epilogue group (named barrier 1 + g) that also returns
-// whether p held on every one of them.
-__device__ __forceinline__ bool group_all(bool p, int g) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred pi, po;\n\t"
-      "setp.ne.u32 pi, %1, 0;\n\t"
-      "bar.red.and.pred po, %2, %3, pi;\n\t"
-      "selp.u32 %0, 1, 0, po;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)p), "r"(1 + g), "n"(kGroupThreads)
-      : "memory");
-  return r != 0;
-}
-
-// The vectors of the surrogate head h in slot: the first layer's context half folded into c1 (one
-// 64-term dot product per hidden unit), the second layer's biases, C_h; by the kGroupThreads
-// threads of a group.
-__device__ __noinline__ void head_vectors(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int gt) {
-  const int u = gt & 127, uu = u & 63;
-  if (gt < 128) {
-    const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
-    const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
-    float acc = (u < 64 ? a.sw.g1_b : a.sw.d1_b)[h * 64 + uu];
+// Entry u (0 .. 127) of the vectors of the surrogate head h in slot: of c1, the first layer's context
+// half folded (a 64-term dot product per hidden unit), and of the second layer's biases and C_h.
+__device__ __noinline__ void head_c1(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int u) {
+  const int uu = u & 63;
+  const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
+  const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
+  float acc = (u < 64 ? a.sw.g1_b : a.sw.d1_b)[h * 64 + uu];
 #pragma unroll
-    for (int kq = 0; kq < 8; ++kq) {
-      const uint4 wv = reinterpret_cast<const uint4*>(w)[kq];
-      const float4 c0 = ctx[2 * kq], c1 = ctx[2 * kq + 1];
-      acc = fmaf(bf16_lo(wv.x), c0.x, fmaf(bf16_hi(wv.x), c0.y, acc));
-      acc = fmaf(bf16_lo(wv.y), c0.z, fmaf(bf16_hi(wv.y), c0.w, acc));
-      acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
-      acc = fmaf(bf16_lo(wv.w), c1.z, fmaf(bf16_hi(wv.w), c1.w, acc));
-    }
-    sm.c1[slot][u] = acc;
-  } else {
-    const float b = (u < 64 ? a.sw.g2_b : a.sw.d2_b)[h * 64 + uu];
-    sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
-    if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
+  for (int kq = 0; kq < 8; ++kq) {
+    const uint4 wv = reinterpret_cast<const uint4*>(w)[kq];
+    const float4 c0 = ctx[2 * kq], c1 = ctx[2 * kq + 1];
+    acc = fmaf(bf16_lo(wv.x), c0.x, fmaf(bf16_hi(wv.x), c0.y, acc));
+    acc = fmaf(bf16_lo(wv.y), c0.z, fmaf(bf16_hi(wv.y), c0.w, acc));
+    acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
+    acc = fmaf(bf16_lo(wv.w), c1.z, fmaf(bf16_hi(wv.w), c1.w, acc));
   }
+  sm.c1[slot][u] = acc;
+}
+__device__ __forceinline__ void head_out(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int u) {
+  const float b = (u < 64 ? a.sw.g2_b : a.sw.d2_b)[h * 64 + (u & 63)];
+  sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
+  if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
 }
 
 struct TcMaps {
@@ -167,9 +156,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     }
     for (int g = 0; g < kTcGroups; ++g) {
       mbar_init(&sm.d1_full[g], 2);  // the MMA commit (or a stand-in) + the item hand-over
-      mbar_init(&sm.h_full[g], kGroupThreads);
+      mbar_init(&sm.h_full[g], 4 * kTcParts);  // a warp each
       mbar_init(&sm.d2_full[g], 1);
-      mbar_init(&sm.taken[g], 1);      // the group has read a tile's item and left its last one
+      mbar_init(&sm.taken[g], 4 * kTcParts);   // every warp has read a mean item
+      mbar_init(&sm.vec_full[g], 4 * kTcParts);
     }
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
@@ -242,18 +232,22 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
           sm.stage_item[st] = it;
           sm.stage_fill[st] = fill;
           sm.stage_head[st] = h;
+          sm.stage_slot[st] = slot;
+          sm.stage_tile[st] = tile;
           mbar_arrive_expect_tx(&sm.full[st], kVTileBytes);
           tma_load_2d(sm.v[st], &maps.v, &sm.full[st], (2 * H + h) * 64, tile * kTcTile);
         }
         __syncwarp();
         tma_k[st] = k;
       } else {
-        const int slot = (it - surr_items) / Tm;
+        const int slot = (it - surr_items) / Tm, tile = it - surr_items - slot * Tm;
         const int h = a.head_ids[m_first + slot];
         if (elect_one()) {
           sm.stage_item[st] = it;
           sm.stage_fill[st] = -1;
           sm.stage_head[st] = h;
+          sm.stage_slot[st] = slot;
+          sm.stage_tile[st] = tile;
           mbar_arrive(&sm.full[st]);
         }
         __syncwarp();
@@ -285,17 +279,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     uint32_t qsur[2];
     int qn = 0;
     uint32_t sur_cnt[kTcGroups] = {0u, 0u};  // surrogate tiles sent to group g
-    int last_kind[kTcGroups] = {-1, -1};        // kind of group g's last tile (1 surrogate, 0 mean)
-    int last_sur[kTcGroups] = {0, 0};           // its index among the group's surrogate tiles
-    // Tile kk may go to its group once the group's previous tile no longer needs what tile kk
-    // overwrites: its second layer has completed (its H lies in the half that tile kk's first
-    // layer writes, and its item was read before), or, for a mean tile, the group has started
-    // it (so it has finished the tile before, whose results lie in that half).
+    uint32_t sec_cnt[kTcGroups] = {0u, 0u};  // their second layers issued
+    uint32_t mean_cnt[kTcGroups] = {0u, 0u}; // mean items sent to group g
+    int last_kind[kTcGroups] = {-1, -1};     // kind of group g's last tile (1 surrogate, 0 mean)
+    // Tile kk may go to its group once the group's previous tile's second layer has been issued
+    // (it reads H, which tile kk's first layer overwrites, and every warp has read the item), or,
+    // for a mean item, once every warp has read it.
     auto group_free = [&](int kk) -> bool {
-      const int gb = kk & 1, jj = kk >> 1;
-      if (jj == 0) return true;
-      if (last_kind[gb] == 1) return mbar_test_wait(&sm.d2_full[gb], (uint32_t)last_sur[gb] & 1);
-      return mbar_test_wait(&sm.taken[gb], (uint32_t)(jj - 1) & 1);
+      const int gb = kk & 1;
+      if (last_kind[gb] < 0) return true;
+      if (last_kind[gb] == 1) return sec_cnt[gb] == sur_cnt[gb];
+      return mbar_test_wait(&sm.taken[gb], (mean_cnt[gb] - 1) & 1);
     };
     unsigned long long t0 = 0;
     for (uint32_t spin = 1;; ++spin) {
@@ -305,9 +299,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
         const bool ready = __shfl_sync(0xffffffffu, (int)mbar_test_wait(&sm.h_full[pb], qsur[0] & 1), 0);
         if (ready) {
           tc_fence_after();
-          // Local tile j of group pb: D2 into the main half (j & 1), H read from the other one.
-          const uint32_t t_main = tmem + pb * 256 + ((qk[0] >> 1) & 1) * 128;
-          const uint32_t t_h = tmem + pb * 256 + (((qk[0] >> 1) & 1) ^ 1) * 128;
+          const uint32_t t_h = tmem + pb * 256, t_main = t_h + 128;
           const uint64_t dg = sdesc_sw128(smem_u32(sm.w2[qfill[0] & 1]));
           const uint64_t dd = sdesc_sw128(smem_u32(sm.w2[qfill[0] & 1] + 64 * 64));
           if (elect_one()) {
@@ -315,11 +307,12 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
             for (int kk = 0; kk < 4; ++kk)  // gamma: hidden units 0..63 = H columns 0..31
               tc_mma_ts(t_main, t_h + 8 * kk, dg + 2 * kk, id2, kk > 0 ? 1u : 0u);
 #pragma unroll
-            for (int kk = 0; kk < 4; ++kk)  // delta: hidden units 64..127 = H columns 32..63
-              tc_mma_ts(t_main + 64, t_h + 32 + 8 * kk, dd + 2 * kk, id2, kk > 0 ? 1u : 0u);
+            for (int kk = 0; kk < 4; ++kk)  // delta: hidden units 64..127 = H columns 64..95
+              tc_mma_ts(t_main + 64, t_h + 64 + 8 * kk, dd + 2 * kk, id2, kk > 0 ? 1u : 0u);
             tc_commit(&sm.d2_full[pb]);
           }
           __syncwarp();
+          ++sec_cnt[pb];
           qk[0] = qk[1];
           qfill[0] = qfill[1];
           qsur[0] = qsur[1];
@@ -341,6 +334,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
           const int it = *reinterpret_cast<volatile int*>(&sm.stage_item[st]);
           const int fill = *reinterpret_cast<volatile int*>(&sm.stage_fill[st]);
           const int head = *reinterpret_cast<volatile int*>(&sm.stage_head[st]);
+          const int item_slot = *reinterpret_cast<volatile int*>(&sm.stage_slot[st]);
+          const int item_tile = *reinterpret_cast<volatile int*>(&sm.stage_tile[st]);
           if (it < 0) {
             feeding = false;
             progress = true;
@@ -351,7 +346,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
             if (fill >= 0) {
               const uint64_t da = sdesc_sw128(smem_u32(sm.v[st]));
               const uint64_t db = sdesc_sw128(smem_u32(sm.w1[fill & 1]));
-              const uint32_t t_main = tmem + b * 256 + ((k >> 1) & 1) * 128;
+              const uint32_t t_main = tmem + b * 256;
               if (elect_one()) {
 #pragma unroll
                 for (int kk = 0; kk < 4; ++kk)  // K = 64 channels: 4 x K16, +32 bytes per step
@@ -367,6 +362,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
             if (elect_one()) {
               sm.acc_item[b] = it;
               sm.acc_head[b] = head;
+              sm.acc_slot[b] = item_slot;
+              sm.acc_tile[b] = item_tile;
               mbar_arrive(&sm.d1_full[b]);  // releases acc_item / acc_head to the group
             }
             __syncwarp();
@@ -383,10 +380,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
               qk[qn] = k;
               qfill[qn] = fill;
               qsur[qn] = sur_cnt[b];
-              last_sur[b] = (int)sur_cnt[b]++;
+              ++sur_cnt[b];
               ++qn;
             }
             last_kind[b] = fill >= 0 ? 1 : 0;
+            if (fill < 0) ++mean_cnt[b];
             ++k;
             progress = true;
           }
@@ -455,9 +453,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     const int g = e / (4 * kTcParts), part = (e % (4 * kTcParts)) >> 2;
     const int gt = tid - 64 - kGroupThreads * g;  // 0 .. kGroupThreads - 1 within the group
     const int quarter = warp & 3;                 // TMEM lanes this warp may access
-    const int row = quarter * 32 + lane;          // token row of the tile = TMEM lane
     const uint32_t t_grp = tmem + ((uint32_t)(quarter * 32) << 16) + g * 256;
-    unsigned char* yrow = reinterpret_cast<unsigned char*>(sm.ys[g]) + row * 128;
+    unsigned char* yblk = reinterpret_cast<unsigned char*>(sm.ys[e]);
     // This warp's share of a row: hidden-unit chunks [g0, g1) of 16 (first layer, H) and
     // output-column chunks [f0, f1) of 16 (second layer, y).
     const int g0 = part_begin(part, 8), g1 = part_begin(part + 1, 8);
@@ -466,52 +463,60 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     bool ok = true;
     // The heads' vectors: all of them now, while the first tile's copies and MMAs run, or with
     // single items (few of a CTA's heads are ever used) each when a tile first needs it.
-    uint32_t ready = 0;  // heads (by slot) whose vectors this group has seen to
+    uint32_t ready = 0;  // heads (by slot) whose vectors this warp can read
+    // A head's vectors by the group's warps: an entry of c1 in lanes 0-15, of the rest in 16-31,
+    // handed over through an mbarrier (a bounded wait, unlike a named barrier).
+    uint32_t n_vec = 0;
+    auto group_vectors = [&](int slot, int h) -> bool {
+      const int u = (4 * part + quarter) * 16 + (lane & 15);
+      if (lane < 16)
+        head_c1(a, sm, slot, h, u);
+      else
+        head_out(a, sm, slot, h, u);
+      ready |= 1u << slot;
+      __syncwarp();
+      if (elect_one()) mbar_arrive(&sm.vec_full[g]);
+      __syncwarp();
+      return mbar_wait_warp(&sm.vec_full[g], n_vec++ & 1, err, abort_flag);
+    };
     if (batch > 1) {
-      for (int sl = 0; sl < n_surr; sl += 2)
-        if (sl + g < n_surr) head_vectors(a, sm, sl + g, a.head_ids[s_first + sl + g], gt);
+      for (int i = tid - 64; i < n_surr * 128; i += kGroupThreads * kTcGroups) {
+        head_c1(a, sm, i >> 7, a.head_ids[s_first + (i >> 7)], i & 127);
+        head_out(a, sm, i >> 7, a.head_ids[s_first + (i >> 7)], i & 127);
+      }
       ready = 0xffffffffu;
       asm volatile("bar.sync 3, %0;" ::"n"(kGroupThreads * kTcGroups) : "memory");
     } else if (g == 0 && first_item < surr_items) {
-      const int sl = first_item / T;
-      head_vectors(a, sm, sl, a.head_ids[s_first + sl], gt);
-      ready = 1u << sl;  // seen by the group behind the barrier below
+      ok = group_vectors(first_item / T, a.head_ids[s_first + first_item / T]);
     }
     for (uint32_t j = 0;; ++j) {
-      ok = group_all(mbar_wait_warp(&sm.d1_full[g], j & 1, err, abort_flag), g);
+      ok = ok && mbar_wait_warp(&sm.d1_full[g], j & 1, err, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const int it = *reinterpret_cast<volatile int*>(&sm.acc_item[g]);
       if (it < 0) break;
       const int h = *reinterpret_cast<volatile int*>(&sm.acc_head[g]);
       const bool surr = it < surr_items;
-      const int tile = surr ? it % T : (it - surr_items) % Tm;  // a mean item spans kMeanRows rows
-      const int slot = surr ? it / T : 0;  // surrogate head slot: its vectors
-      if (surr && !((ready >> slot) & 1u)) {
-        head_vectors(a, sm, slot, h, gt);
-        ready |= 1u << slot;
-        group_all(true, g);
-      }
+      const int tile = *reinterpret_cast<volatile int*>(&sm.acc_tile[g]);  // a mean item spans kMeanRows rows
+      const int slot = *reinterpret_cast<volatile int*>(&sm.acc_slot[g]);  // surrogate head slot: its vectors
+      if (surr && !((ready >> slot) & 1u) && !group_vectors(slot, h)) break;
       const float* c1 = sm.c1[slot];
       const float* b2 = sm.b2[slot];
       const float* cx = sm.cx[slot];
-      // This tile's halves of the group's columns: D1 / D2 in the main one (j & 1), H in the
-      // first 64 columns of the other.
-      const uint32_t t_acc = t_grp + (j & 1) * 128;
-      const uint32_t t_h = t_grp + ((j & 1) ^ 1) * 128;
+      const uint32_t t_d1 = t_grp, t_d2 = t_grp + 128;
       if (surr) {
         // H = 2 GELU(D1 + c1) as bf16 pairs (the factor 2 is exact in bf16 and is taken out
-        // of the second layer's results): chunk c of 16 hidden units (D1 columns 16 c ..)
-        // into H columns 8 c .. + 8.  Each chunk's TMEM load is in flight while the chunk
-        // before it is computed.
+        // of the second layer's results): chunk c of 16 hidden units (D1 columns 16 c ..) into 8
+        // columns at the start of this warp's own D1 columns (64 part ..), which it has read by
+        // then.  Each chunk's TMEM load is in flight while the chunk before it is computed.
         float vb[2][16];
-        tmem_ld16(t_acc + 16 * g0, vb[0]);
+        tmem_ld16(t_d1 + 16 * g0, vb[0]);
 #pragma unroll
         for (int i = 0; i < kMaxGChunks; ++i) {
           const int c = g0 + i;
           if (c >= g1) break;
           tmem_wait_ld();
-          if (c + 1 < g1) tmem_ld16(t_acc + 16 * (c + 1), vb[(i + 1) & 1]);
+          if (c + 1 < g1) tmem_ld16(t_d1 + 16 * (c + 1), vb[(i + 1) & 1]);
           uint32_t hw[8];
 #pragma unroll
           for (int q = 0; q < 8; ++q) {
@@ -519,21 +524,26 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
             const float2 x = gelu2_as2(fadd2(make_float2(vb[i & 1][2 * q], vb[i & 1][2 * q + 1]), cc));
             hw[q] = pack_bf16x2(x.x, x.y);
           }
-          tmem_st8(t_h + 8 * c, hw);
+          tmem_st8(t_d1 + 64 * part + 8 * i, hw);
         }
         tmem_wait_st();
         tc_fence_before();
-        mbar_arrive(&sm.h_full[g]);
+        __syncwarp();
+        if (elect_one()) {
+          mbar_arrive(&sm.h_full[g]);
+          tma_store_wait_read<0>();  // the last tile's store has read the staging block
+        }
+        __syncwarp();
         ok = mbar_wait_warp(&sm.d2_full[g], sj & 1, err, abort_flag);
+        if (!ok) break;
         ++sj;
       }
       if (!surr) {
         // Broadcast(mean of V_h) straight to Y (no staging: a store pipeline two tiles deep
         // per SM would hold these pure-write tiles back): eight threads per row, each a 16-byte
         // chunk, so that a warp writes whole 128-byte rows.
-        ok = group_all(ok, g);
-        if (!ok) break;
-        if (gt == 0) mbar_arrive(&sm.taken[g]);  // every thread has read this tile's item
+        __syncwarp();
+        if (elect_one()) mbar_arrive(&sm.taken[g]);  // this warp has read the item
         const int jc = gt & 7;
         const float4 m0 = reinterpret_cast<const float4*>(a.mean_v + h * 64)[2 * jc];
         const float4 m1 = reinterpret_cast<const float4*>(a.mean_v + h * 64)[2 * jc + 1];
@@ -545,11 +555,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
         }
         continue;
       }
-      // The staging buffer is free once the previous store from it has read it.
-      if (gt == 0) tma_store_wait_read<0>();
-      ok = group_all(ok, g);
-      if (!ok) break;
-      if (gt == 0) mbar_arrive(&sm.taken[g]);  // every thread has read this tile's item
       {
         // y = C + sigma(D2g + b2g) (.) (D2d + b2d) for chunk c of 16 output columns, from
         // D2' = 2 D2: sigma(u) = 1 / (1 + 2^(-log2(e) u)) with the exponent
@@ -561,8 +566,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
           const int c = f0 + i;
           if (c >= f1) break;
           float og[16], od[16];
-          tmem_ld16(t_acc + 16 * c, og);
-          tmem_ld16(t_acc + 64 + 16 * c, od);
+          tmem_ld16(t_d2 + 16 * c, og);
+          tmem_ld16(t_d2 + 64 + 16 * c, od);
           tmem_wait_ld();
           uint32_t yw[8];
 #pragma unroll
@@ -581,22 +586,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
             yw[q] = pack_bf16x2(y2.x, y2.y);
           }
 #pragma unroll
-          for (int q = 0; q < 2; ++q) {  // 16-byte chunk jc of the row sits at chunk jc ^ (row & 7)
-            const int jc = 2 * c + q;
-            *reinterpret_cast<uint4*>(yrow + ((jc ^ (row & 7)) << 4)) =
+          for (int q = 0; q < 2; ++q) {  // 64-byte swizzle: chunk jc of row r sits at jc ^ ((r >> 1) & 3)
+            const int jc = 2 * i + q;
+            *reinterpret_cast<uint4*>(yblk + lane * 64 + ((jc ^ ((lane >> 1) & 3)) << 4)) =
                 make_uint4(yw[4 * q], yw[4 * q + 1], yw[4 * q + 2], yw[4 * q + 3]);
           }
         }
         tc_fence_before();
       }
       fence_proxy_async_smem();
-      group_all(true, g);
-      if (gt == 0) {
-        tma_store_2d(&maps.y, sm.ys[g], h * 64, tile * kTcTile);
+      __syncwarp();
+      if (elect_one()) {
+        tma_store_2d(&maps.y, yblk, h * 64 + 16 * f0, tile * kTcTile + quarter * 32);
         tma_store_commit();
       }
+      __syncwarp();
     }
-    if (gt == 0) tma_store_wait_all();
+    if (elect_one()) tma_store_wait_all();
+    __syncwarp();
   }
   tc_fence_before();
   __syncthreads();
@@ -634,7 +641,7 @@ cudaError_t launch_cheap_heads_tc(const HeadAttnArgs& a, int num_sms, cudaStream
   if ((e = make_tmap_bf16_2d(&maps.v, a.qkv, 3 * H * 64, (uint64_t)a.N, 3 * H * 64, 64, kTcTile)) !=
       cudaSuccess)
     return e;
-  if ((e = make_tmap_bf16_2d(&maps.y, a.y, H * 64, (uint64_t)a.N, H * 64, 64, kTcTile)) != cudaSuccess)
+  if ((e = make_tmap_bf16_2d(&maps.y, a.y, H * 64, (uint64_t)a.N, H * 64, 32, 32, 64)) != cudaSuccess)
     return e;
   // Layer-1 weights [H][64][128]: the value half is columns 0..63; layer 2 [H][64][64].
   if ((e = make_tmap_bf16_2d(&maps.g1, a.sw.g1_w, 128, H * 64, 128, 64, 64)) != cudaSuccess) return e;
