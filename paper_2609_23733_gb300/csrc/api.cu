@@ -250,6 +250,7 @@ vp_status check_qk(const vp_qk_options* qk, const vp_dims* dm, int* max_pos) {
 struct QkArgs {
   const vp_qk_options* o;
   const float2* table;
+  int npos;                  // positions of the table
   const int32_t* tok_index;  // token of each row (merged tokens), or NULL
 };
 
@@ -265,6 +266,7 @@ void set_qk(LinearArgs& la, const QkArgs* qk, int D) {
   la.qk_eps = o.norm_eps;
   if (o.rope) {
     la.rope_cs = qk->table;
+    la.rope_npos = qk->npos;
     la.tok_per_view = o.tokens_per_view;
     la.patch_start = o.patch_start;
     la.grid_w = o.grid_w;
@@ -637,7 +639,7 @@ vp_status vp_moh_global_attention(const vp_dims* dims, const vp_bf16* x, const v
   float2* rope = reinterpret_cast<float2*>(p);
   p += align_up(kRopeTableBytes);
   if (qk && qk->rope) VP_TRY(from_cuda(launch_rope_table(max_pos, qk->rope_base, rope, st)));
-  const QkArgs qa{qk, rope, nullptr};
+  const QkArgs qa{qk, rope, max_pos + 1, nullptr};
   __nv_bfloat16* qkv = reinterpret_cast<__nv_bfloat16*>(p);
   p += align_up(N * 3 * D * 2);
   __nv_bfloat16* y = reinterpret_cast<__nv_bfloat16*>(p);
@@ -697,6 +699,7 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
   float2* rope = reinterpret_cast<float2*>(p);
   p += align_up(kRopeTableBytes);
   const vp_qk_options* rope_built = nullptr;  // the options the table was last built for
+  int rope_npos = 1;
   // LayerNorm scratch (see ln_scratch_bytes).  LN1 is folded into the QKV projection, which
   // then reads the raw residual stream; its row statistics come from the kernel that last
   // wrote the stream (the previous block's FFN-down, or a statistics pass for the first
@@ -756,6 +759,7 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
       int max_pos = 0;
       VP_TRY(check_qk(w.qk, dims, &max_pos));
       VP_TRY(from_cuda(launch_rope_table(max_pos, w.qk->rope_base, rope, st)));
+      rope_npos = max_pos + 1;
       rope_built = w.qk;
     }
     const int32_t* fm = force_modes ? force_modes + (size_t)l * dims->H : nullptr;
@@ -778,14 +782,14 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
                                          cudaMemcpyDeviceToDevice, st)));
       vp_dims dm = *dims;
       dm.N = g.Np;
-      const QkArgs qm{w.qk, rope, ms.dst_tok};
+      const QkArgs qm{w.qk, rope, rope_npos, ms.dst_tok};
       VP_TRY(run_layer(&dm, ms.xm, w.w_qkv, w.b_qkv, w.w_o, w.b_o, nullptr, nullptr, &w.router,
                        &w.surrogate, fm, merged_out, qkv, y, s_l, sa_l, m_l, sc, st, nullptr, &qm));
       // unmerge, X_attn = X + LS1 (.) A, and (4)'s Z~ = LN2(X_attn) in one pass
       VP_TRY(from_cuda(launch_unmerge_ln(dims->N, D, ms.assign, merged_out, w.ls1, w.ln2_g,
                                          w.ln2_b, ln_eps, x, zt, st)));
     } else {
-      const QkArgs qa{w.qk, rope, nullptr};
+      const QkArgs qa{w.qk, rope, rope_npos, nullptr};
       // (1)-(3) X <- X + LS1 (Y W_O + b_O) in place, Y the routed attention of LN1(X)
       const LnFold fold{part, cq, ln_eps};
       VP_TRY(run_layer(dims, x, reinterpret_cast<const vp_bf16*>(wq), bq, w.w_o, w.b_o, w.ls1, x,

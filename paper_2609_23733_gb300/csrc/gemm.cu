@@ -76,7 +76,7 @@ struct GemmParams {
   const float* kn_b;
   float qk_eps;
   const float2* rope_cs;
-  int tok_per_view, patch_start, grid_w;
+  int rope_npos, tok_per_view, patch_start, grid_w;
   const int32_t* tok_index;
   const int32_t* skip_ids;
   const int32_t* skip_off;
@@ -100,7 +100,7 @@ __device__ __forceinline__ TileUnit tile_unit(int u, int full_units, int n_tiles
 
 // kSkip: the instance that leaves K-blocks out (GemmParams::skip_ids); the other instance has
 // none of that bookkeeping.
-template <bool kSkip, int kEpiWarps>
+template <bool kSkip, int kEpiWarps, bool kQk = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 const __grid_constant__ CUtensorMap tmap_b,
@@ -418,7 +418,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         }
         ++nst;
       };
-      if (kParts == 2 && prm.qk_cols > 0 && pcol0 < prm.qk_cols) {
+      if (kQk && pcol0 < prm.qk_cols) {
         // Q or K columns of a QKV projection with qk-norm and / or 2-D RoPE: whole heads
         // (64 columns, two chunks) at a time.
         const bool is_q = pcol0 < (prm.qk_cols >> 1);
@@ -473,10 +473,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
           if (prm.rope_cs) {  // channels [0, 32) turn with the row, [32, 64) with the column
 #pragma unroll
             for (int ax = 0; ax < 2; ++ax) {
-              const float4* cs = reinterpret_cast<const float4*>(prm.rope_cs + (size_t)(ax ? px : py) * 16);
+              const float4* cs = reinterpret_cast<const float4*>(prm.rope_cs) + (ax ? px : py);
 #pragma unroll
               for (int q = 0; q < 8; ++q) {  // frequencies 2q, 2q + 1: (cos, sin) pairs
-                const float4 t4 = cs[q];
+                const float4 t4 = cs[q * prm.rope_npos];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                   const int i = 32 * ax + 2 * q + e;
@@ -517,7 +517,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
           }
           // Bias, GELU, LayerScale and residual on column pairs (packed f32x2 arithmetic).
           bias_fold(x, col0);
-          if (prm.act == VP_ACT_GELU) {
+          if (!kQk && prm.act == VP_ACT_GELU) {
 #pragma unroll
             for (int k = 0; k < 16; ++k) {
               const float2 gk = gelu_as2(make_float2(x[2 * k], x[2 * k + 1]));
@@ -525,7 +525,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
               x[2 * k + 1] = gk.y;
             }
           }
-          if (prm.scale) {
+          if (!kQk && prm.scale) {
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
               const float4 s4 = reinterpret_cast<const float4*>(&sm.vec[1][col0 - t.n0])[q];
@@ -537,7 +537,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
               x[4 * q + 3] = a1.y;
             }
           }
-          if (prm.residual) {  // rows and columns past the edge were filled with zeros
+          if (!kQk && prm.residual) {  // rows and columns past the edge were filled with zeros
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const uint4 ru = *reinterpret_cast<const uint4*>(brow + (((4 * (cc & 1) + q) ^ (lane & 7)) << 4));
@@ -551,7 +551,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
               }
             }
           }
-          if (kParts == 2 && prm.part_out) {  // chunk mean and M2 (two passes over registers)
+          if (!kQk && kParts == 2 && prm.part_out) {  // chunk mean and M2 (two passes over registers)
             float2 s2 = make_float2(0.f, 0.f);
 #pragma unroll
             for (int k = 0; k < 16; ++k) s2 = fadd2(s2, make_float2(x[2 * k], x[2 * k + 1]));
@@ -572,7 +572,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         if (cc + 2 == 2 * n_grp) release_acc();  // the last chunk is in registers
       }
       const int pcol = pcol0;  // this thread's 128-column block
-      if (kParts == 2 && prm.part_out && row_ok && pcol < N) {
+      if (!kQk && kParts == 2 && prm.part_out && row_ok && pcol < N) {
         const float mb = 0.25f * (cmean[0] + cmean[1] + cmean[2] + cmean[3]);
         float m2 = cm2[0] + cm2[1] + cm2[2] + cm2[3];
 #pragma unroll
@@ -593,7 +593,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
   }
 }
 
-// RoPE angles in double precision: table[p][i] = (cos, sin)(p base^(-i / 16)).
+// RoPE angles in double precision: (cos, sin)(p base^(-i / 16)) at table[i / 2][p][i % 2]: the rows of
+// a warp stand at neighbouring positions, so its 16-byte loads of one frequency pair lie side by
+// side (with the pairs of a position side by side, a load took 32 cache lines and the epilogue set
+// the time: QKV with qk-norm at 43,968 tokens 189 -> 163 us).
 __global__ void rope_table_kernel(int max_pos, double base, float2* table) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int p = k >> 4, i = k & 15;
@@ -602,7 +605,7 @@ __global__ void rope_table_kernel(int max_pos, double base, float2* table) {
   pdl_wait();
   pdl_launch();
   if (k >= (max_pos + 1) * 16) return;
-  table[k] = make_float2((float)cs, (float)sn);
+  table[((i >> 1) * (max_pos + 1) + p) * 2 + (i & 1)] = make_float2((float)cs, (float)sn);
 }
 
 }  // namespace
@@ -672,7 +675,7 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
   GemmParams prm{a.M,     a.N,   a.K,   a.bias,      a.act,  a.scale,   a.residual,
                  a.out,   a.err, a.ln_part, a.ln_c, a.ln_eps, a.part_out,
                  qk ? a.qk_cols : 0, a.qn_g, a.qn_b, a.kn_g, a.kn_b, a.qk_eps, a.rope_cs,
-                 a.tok_per_view, a.patch_start, a.grid_w, a.tok_index, a.skip_ids, a.skip_off,
+                 a.rope_npos, a.tok_per_view, a.patch_start, a.grid_w, a.tok_index, a.skip_ids, a.skip_off,
                  full_units, units};
   const int grid = 2 * min(pairs_max, units);
   const int smem = (int)sizeof(GemmSmem);
@@ -690,7 +693,8 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
   // 1,024 with residual 15.4 -> 12.2 us).  Eight elsewhere (128 columns, two blocks, so that the
   // next tile's residual loads start earlier: 137,400 x 1,024 with residual 183 us against 189,
   // x 3,072 454 against 462); qk-norm and part_out need a thread to hold whole heads or blocks.
-  const bool sixteen = !a.part_out && !qk && (a.act == VP_ACT_GELU || units <= pairs_max);
+  const bool sixteen = !a.part_out && (a.act == VP_ACT_GELU || units <= pairs_max);
+  if (qk) return launch(gemm_kernel<false, 8, true>, 8);
   if (a.skip_ids) return sixteen ? launch(gemm_kernel<true, 16>, 16) : launch(gemm_kernel<true, 8>, 8);
   return sixteen ? launch(gemm_kernel<false, 16>, 16) : launch(gemm_kernel<false, 8>, 8);
 }

@@ -188,7 +188,8 @@ struct LinearArgs {
   const float* kn_g;
   const float* kn_b;
   float qk_eps;
-  const float2* rope_cs;  // NULL: no RoPE
+  const float2* rope_cs;  // NULL: no RoPE; launch_rope_table's layout for rope_npos positions
+  int rope_npos;
   int tok_per_view, patch_start, grid_w;
   const int32_t* tok_index;  // RoPE: token index of output row r (merged tokens), or NULL (r)
   // K-blocks left out (W_O with mean heads folded into its bias): the 64-column blocks kb =
@@ -214,7 +215,7 @@ cudaError_t launch_ln_partials(int M, int D, const __nv_bfloat16* x, float2* par
 // Wp = W diag(g) (bf16), c[o] = sum_k Wp[o][k] (of the bf16 Wp), bp[o] = b[o] + sum_k W[o][k] beta[k]
 // (b NULL: 0).  K % 256 == 0, K <= 4096.  weights_ready: no kernel just before writes W, g, beta or b,
 // and none reads the outputs any more (see ln_fold_kernel).
-// cos / sin of p * base^(-i / 16), p = 0 .. max_pos, i = 0 .. 15: table [max_pos + 1][16].
+// cos / sin of p * base^(-i / 16), p = 0 .. max_pos, i = 0 .. 15: table [i / 2][max_pos + 1][i % 2].
 cudaError_t launch_rope_table(int max_pos, float base, float2* table, cudaStream_t st);
 cudaError_t launch_ln_fold_weights(int Nout, int K, const __nv_bfloat16* W, const float* g,
                                    const float* beta, const float* b, __nv_bfloat16* Wp,
