@@ -109,6 +109,25 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, u
   return __all_sync(0xffffffffu, ok);
 }
 
+// Two barriers tested together, so that their round trips overlap.
+__device__ __forceinline__ bool mbar_wait2_warp(uint64_t* bar0, uint32_t parity0, uint64_t* bar1,
+                                                uint32_t parity1, unsigned int* err,
+                                                volatile int* abort_flag) {
+  const bool t0 = mbar_test_wait(bar0, parity0), t1 = mbar_test_wait(bar1, parity1);
+  bool ok = t0 || mbar_wait(bar0, parity0, err, abort_flag);
+  ok = ok && (t1 || mbar_wait(bar1, parity1, err, abort_flag));
+  return __all_sync(0xffffffffu, ok);
+}
+
+// Counter increment that releases what this CTA wrote before (through a __syncthreads before it) and
+// acquires what the CTAs counted before wrote (through a __syncthreads after it): one thread's
+// acq_rel atomic instead of a fence in every thread.
+__device__ __forceinline__ unsigned int atomic_inc_acq_rel(unsigned int* p) {
+  unsigned int old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(p) : "memory");
+  return old;
+}
+
 // ---------------------------------------------------------------- TMA
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");

@@ -119,12 +119,12 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
   if (tid == 0) {
     for (int s = 0; s < kPoolTcStages; ++s) {
       mbar_init(&sm.q_full[s], 1);
-      mbar_init(&sm.q_empty[s], 128);
+      mbar_init(&sm.q_empty[s], 4);  // a token warp each
     }
     mbar_init(&sm.wu_full, 1);
     for (int b = 0; b < kPoolAccBufs; ++b) {
       mbar_init(&sm.acc_full[b], 1);
-      mbar_init(&sm.acc_empty[b], 128);
+      mbar_init(&sm.acc_empty[b], 4);
     }
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
@@ -156,9 +156,9 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
   const uint32_t tmem = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
 
   float Mx = -INFINITY, lsum = 0.f;  // epilogue threads: this thread's tokens
-  float acc[64];
+  float2 acc[32];
 #pragma unroll
-  for (int c = 0; c < 64; ++c) acc[c] = 0.f;
+  for (int c = 0; c < 32; ++c) acc[c] = make_float2(0.f, 0.f);
 
   if (warp == 4) {
     // ------------------------------------------------------------ TMA producer
@@ -225,8 +225,8 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
       const int st = i % kPoolTcStages, ab = i % kPoolAccBufs;
       // The tile's accumulator, and its Q rows in shared memory (read below by these threads:
       // they wait on the TMA's barrier themselves rather than rely on the MMA's).
-      ok = mbar_wait_warp(&sm.acc_full[ab], (i / kPoolAccBufs) & 1, err, abort_flag) &&
-           mbar_wait_warp(&sm.q_full[st], (i / kPoolTcStages) & 1, err, abort_flag);
+      ok = mbar_wait2_warp(&sm.acc_full[ab], (i / kPoolAccBufs) & 1, &sm.q_full[st],
+                           (i / kPoolTcStages) & 1, err, abort_flag);
       if (!ok) break;
       tc_fence_after();
       float e2x = 0.f, e2y = 0.f;
@@ -238,7 +238,8 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
         tmem_wait_ld();
         if (qtr == 3) {  // the accumulator is in registers: back to the MMA warp
           tc_fence_before();
-          mbar_arrive(&sm.acc_empty[ab]);
+          __syncwarp();
+          if (elect_one()) mbar_arrive(&sm.acc_empty[ab]);
         }
         float2 pe = make_float2(0.f, 0.f);
 #pragma unroll
@@ -263,7 +264,7 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
           const float sc_ = __expf(Mx - e);
           lsum *= sc_;
 #pragma unroll
-          for (int c = 0; c < 64; ++c) acc[c] *= sc_;
+          for (int c = 0; c < 32; ++c) acc[c] = fmul2(acc[c], make_float2(sc_, sc_));
           Mx = e;
         }
         const float p = __expf(e - Mx);
@@ -275,8 +276,8 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
           const uint32_t w4[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            acc[8 * j + 2 * k] = fmaf(p, bf16_lo(w4[k]), acc[8 * j + 2 * k]);
-            acc[8 * j + 2 * k + 1] = fmaf(p, bf16_hi(w4[k]), acc[8 * j + 2 * k + 1]);
+            acc[4 * j + k] = ffma2(make_float2(p, p), make_float2(bf16_lo(w4[k]), bf16_hi(w4[k])),
+                                   acc[4 * j + k]);
           }
         }
       }
@@ -284,8 +285,9 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
       // are ordered before the async-proxy writes that refill it.  Without the fence the release
       // can overtake loads still in flight: a version with a two-stage ring gave q_pool values
       // up to 3 % off in repeated runs.
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      mbar_arrive(&sm.q_empty[st]);
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (elect_one()) mbar_arrive(&sm.q_empty[st]);
     }
   }
   // Merge the 128 token threads' partials: the CTA maximum, then scaled sums of l and sum p q.
@@ -303,16 +305,17 @@ __global__ void __launch_bounds__(kPoolTcThreads, kPoolCtasPerSm)
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
 #pragma unroll
-    for (int c = 0; c < 64; ++c) {
-      float v = acc[c] * f;
+    for (int c = 0; c < 32; ++c) {
+      float2 v = fmul2(acc[c], make_float2(f, f));
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      for (int o = 16; o > 0; o >>= 1)
+        v = fadd2(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, o), __shfl_xor_sync(0xffffffffu, v.y, o)));
       acc[c] = v;
     }
     if (lane == 0) {
       sm.red_l[warp] = l;
 #pragma unroll
-      for (int c = 0; c < 64; ++c) sm.red_acc[warp][c] = acc[c];
+      for (int c = 0; c < 32; ++c) *reinterpret_cast<float2*>(&sm.red_acc[warp][2 * c]) = acc[c];
     }
   }
   __syncthreads();
@@ -364,6 +367,22 @@ union KeySmem {
   float part[kKeySplitMax * kKeyPartial];
 };
 
+// The factors exp(m_s - max m) of n partials (n <= 64, m at the start of each stride of p) by one warp,
+// f[s] = -1 for a partial without a finite maximum (left out of the sums); returns max m.
+static_assert(kPoolSplitMax <= 64 && kKeySplitMax <= 64, "two partials per lane");
+template <typename F>
+__device__ __forceinline__ float split_factors(const float* p, int stride, int n, float* f, F exp_of) {
+  const int lane = lane_id();
+  const float m0 = lane < n ? p[lane * stride] : -INFINITY;
+  const float m1 = lane + 32 < n ? p[(lane + 32) * stride] : -INFINITY;
+  float mx = fmaxf(m0, m1);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane < n) f[lane] = m0 == -INFINITY ? -1.f : exp_of(m0 - mx);
+  if (lane + 32 < n) f[lane + 32] = m1 == -INFINITY ? -1.f : exp_of(m1 - mx);
+  return mx;
+}
+
 // n floats of another CTA's making (L2) into shared memory by the whole CTA, all loads in flight.
 __device__ __forceinline__ void stage_floats(float* dst, const float* src, int n) {
 #pragma unroll 8
@@ -382,7 +401,7 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
   const float beta = a.beta ? a.beta[h] : 1.f;
   const float cscale = beta * 0.125f * kLog2e;  // beta / sqrt(64), in log2 units
   __shared__ KeySmem sk;
-  __shared__ float s_q[64];
+  __shared__ float s_q[64], s_f[kKeySplitMax], s_mx;
   pdl_wait();
   pdl_launch();
   int t0, t1;
@@ -402,21 +421,20 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
     }
   };
   if (t0 < t1) load_batch(t0);
-  // q_pool from the pooling's partials: threads 0-63, a channel each, splits in order.
+  // q_pool from the pooling's partials: the factors by a warp, then threads 0-63, a channel each,
+  // splits in order.
   stage_floats(sk.pool, sc.pool_part + (size_t)h * kPoolSplitMax * kPoolPartial, pool_split * kPoolPartial);
   __syncthreads();
+  if (tid < 32) split_factors(sk.pool, kPoolPartial, pool_split, s_f, [](float x) { return __expf(x); });
+  __syncthreads();
   if (tid < 64) {
-    const float* pp = sk.pool;
-    float Mx = -INFINITY;
-    for (int s = 0; s < pool_split; ++s) Mx = fmaxf(Mx, pp[s * kPoolPartial]);
     float acc = 0.f, l = 0.f;
 #pragma unroll 4
     for (int s = 0; s < pool_split; ++s) {
-      const float ms = pp[s * kPoolPartial];
-      if (ms == -INFINITY) continue;
-      const float f = __expf(ms - Mx);
-      l += f * pp[s * kPoolPartial + 1];
-      acc += f * pp[s * kPoolPartial + 2 + tid];
+      const float f = s_f[s];
+      if (f < 0.f) continue;
+      l += f * sk.pool[s * kPoolPartial + 1];
+      acc += f * sk.pool[s * kPoolPartial + 2 + tid];
     }
     const float qp = acc / l;
     s_q[tid] = qp;
@@ -477,7 +495,8 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
       }
     }
   }
-  // Combine the 32 row groups of the CTA: threads 0-63, a channel each, groups in order.
+  // Combine the 32 row groups of the CTA: the factors by a warp, then threads 0-63, a channel each,
+  // groups in order.
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     sk.rows.acc[g][8 * part + i] = accv[i];
@@ -488,50 +507,51 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
     sk.rows.l[g] = l;
   }
   __syncthreads();
+  if (tid < 32) {
+    const float mx = split_factors(sk.rows.m, 1, 32, s_f, [](float x) { return fast_exp2(x); });
+    if (tid == 0) s_mx = mx;
+  }
+  __syncthreads();
   float* kp = sc.key_part + ((size_t)h * kKeySplitMax + split) * kKeyPartial;
   if (tid < 64) {
-    float Mx = -INFINITY;
-#pragma unroll
-    for (int i = 0; i < 32; ++i) Mx = fmaxf(Mx, sk.rows.m[i]);
     float acc = 0.f, sum = 0.f, ll = 0.f;
 #pragma unroll 8
     for (int i = 0; i < 32; ++i) {
       sum += sk.rows.sum[i][tid];
-      if (sk.rows.m[i] == -INFINITY) continue;
-      const float f = fast_exp2(sk.rows.m[i] - Mx);
+      const float f = s_f[i];
+      if (f < 0.f) continue;
       acc += f * sk.rows.acc[i][tid];
       ll += f * sk.rows.l[i];
     }
     kp[2 + tid] = acc;
     kp[2 + 64 + tid] = sum;
     if (tid == 0) {
-      kp[0] = Mx;
+      kp[0] = s_mx;
       kp[1] = ll;
     }
   }
   __shared__ int s_last;
-  __threadfence();
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&sc.counters[kMaxHeads + h], 1u) == (unsigned)(n_split - 1));
+  if (tid == 0) s_last = (atomic_inc_acq_rel(&sc.counters[kMaxHeads + h]) == (unsigned)(n_split - 1));
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   // Last CTA of head h: saliency, context, mean of V, mode.
   stage_floats(sk.part, sc.key_part + (size_t)h * kKeySplitMax * kKeyPartial, n_split * kKeyPartial);
   __syncthreads();
+  if (tid < 32) {
+    const float mx = split_factors(sk.part, kKeyPartial, n_split, s_f, [](float x) { return fast_exp2(x); });
+    if (tid == 0) s_mx = mx;
+  }
+  __syncthreads();
   if (tid < 64) {
-    const float* pp = sk.part;
-    float Mx = -INFINITY;
-#pragma unroll 4
-    for (int s = 0; s < n_split; ++s) Mx = fmaxf(Mx, pp[s * kKeyPartial]);
+    const float Mx = s_mx;
     float acc = 0.f, sum = 0.f, ll = 0.f;
 #pragma unroll 4
     for (int s = 0; s < n_split; ++s) {
-      const float* q2 = pp + s * kKeyPartial;
+      const float* q2 = sk.part + s * kKeyPartial;
       sum += q2[2 + 64 + tid];
-      const float ms = q2[0];
-      if (ms == -INFINITY) continue;
-      const float f = fast_exp2(ms - Mx);
+      const float f = s_f[s];
+      if (f < 0.f) continue;
       ll += f * q2[1];
       acc += f * q2[2 + tid];
     }
@@ -558,13 +578,12 @@ __global__ void __launch_bounds__(kKeyThreads) router_keys_kernel(RouterArgs a, 
       if (a.modes_out) a.modes_out[h] = mode;
     }
   }
-  // The last head to finish groups all heads by mode.
-  __threadfence();
+  // In a layer, the last head to finish groups all heads by mode.
+  if (!a.head_counters) return;
   __syncthreads();
-  if (tid == 0) s_last = (atomicAdd(&sc.counters[2 * kMaxHeads], 1u) == (unsigned)(H - 1));
+  if (tid == 0) s_last = (atomic_inc_acq_rel(&sc.counters[2 * kMaxHeads]) == (unsigned)(H - 1));
   __syncthreads();
   if (!s_last) return;
-  __threadfence();
   if (tid < 32) bin_heads_warp(H, sc.modes, sc.head_ids, sc.offsets);
 }
 
@@ -584,18 +603,27 @@ __global__ void __launch_bounds__(256) router_r_kernel(RouterArgs a, RouterScrat
   for (int i = 0; i < 8; ++i) q[i] = __ldcg(sc.q_pool + h * 64 + 8 * part + i) * cscale;
   const float Mx = __ldcg(sc.key_stats + 2 * h), inv = 1.f / __ldcg(sc.key_stats + 2 * h + 1);
   const __nv_bfloat16* kb = a.qkv + (size_t)(H + h) * kHeadDim + 8 * part;
-  for (int base = blockIdx.x * 32; base < N; base += gridDim.x * 32) {  // uniform bound
-    const int row = base + g;
-    const bool valid = row < N;
-    const uint4 kk = *reinterpret_cast<const uint4*>(kb + (size_t)(valid ? row : 0) * row_pitch);
-    const uint32_t kw[4] = {kk.x, kk.y, kk.z, kk.w};
-    float dot = 0.f;
+  // Four rows per group of eight lanes in flight (one at a time the loads' latency set the time:
+  // 17 us for 16 heads at 10,992 tokens, now 12).
+  for (int base = blockIdx.x * 128; base < N; base += gridDim.x * 128) {  // uniform bound
+    uint4 kk[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) dot += q[2 * i] * bf16_lo(kw[i]) + q[2 * i + 1] * bf16_hi(kw[i]);
-    dot += __shfl_xor_sync(0xffffffffu, dot, 1);
-    dot += __shfl_xor_sync(0xffffffffu, dot, 2);
-    dot += __shfl_xor_sync(0xffffffffu, dot, 4);
-    if (valid && part == 0) a.r_out[(size_t)h * N + row] = fast_exp2(dot - Mx) * inv;
+    for (int u = 0; u < 4; ++u) {
+      const int row = base + 32 * u + g;
+      kk[u] = *reinterpret_cast<const uint4*>(kb + (size_t)(row < N ? row : 0) * row_pitch);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int row = base + 32 * u + g;
+      const uint32_t kw[4] = {kk[u].x, kk[u].y, kk[u].z, kk[u].w};
+      float dot = 0.f;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) dot += q[2 * i] * bf16_lo(kw[i]) + q[2 * i + 1] * bf16_hi(kw[i]);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 1);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 2);
+      dot += __shfl_xor_sync(0xffffffffu, dot, 4);
+      if (row < N && part == 0) a.r_out[(size_t)h * N + row] = fast_exp2(dot - Mx) * inv;
+    }
   }
 }
 
@@ -703,7 +731,9 @@ cudaError_t launch_router(const RouterArgs& a, const RouterScratch& sc, int num_
                  dim3(pool_split, a.H), kPoolTcThreads, smem, st, tq, tw, tu, a, sc, pool_split);
   prof_after(st);
   if (e != cudaSuccess) return e;
-  int key_split = (4 * num_sms + a.H - 1) / a.H;
+  // One wave of two CTAs per SM (105 registers): with twice the CTAs the second wave repeated the
+  // set-up (q_pool, combine; about 6 us).
+  int key_split = 2 * num_sms / a.H;
   key_split = max(1, min(min(key_split, kKeySplitMax), (a.N + 255) / 256));
   prof_before(VP_KERNEL_ROUTER_KEYS, st);
   e = launch_pdl(router_keys_kernel, dim3(key_split, a.H), kKeyThreads, 0, st, a, sc, pool_split,
@@ -711,7 +741,7 @@ cudaError_t launch_router(const RouterArgs& a, const RouterScratch& sc, int num_
   prof_after(st);
   if (e != cudaSuccess) return e;
   if (a.r_out) {
-    int blocks = max(1, min((a.N + 31) / 32, (2 * num_sms + a.H - 1) / a.H));
+    int blocks = max(1, min((a.N + 127) / 128, 4 * num_sms / a.H));
     prof_before(VP_KERNEL_ROUTER_R, st);
     e = launch_pdl(router_r_kernel, dim3(blocks, a.H), 256, 0, st, a, sc);
     prof_after(st);
