@@ -132,7 +132,7 @@ def _p(t):
     if t is None:
         return None
     if isinstance(t, torch.Tensor):
-        if t.device.type != "cuda":
+        if not t.is_cuda:
             raise ValueError("device tensors are required (the library has no CPU path)")
         if not t.is_contiguous():
             raise ValueError("tensors must be contiguous")
@@ -150,8 +150,11 @@ def _host_p(t):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    """The cudaStream_t of ``stream``, or of the current stream of the current device (read raw: a
+    torch.cuda.Stream object per call costs more than a small kernel's launch)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def dims(N, H=16, d=64, L=64, tau_low=0.01, tau_high=0.20, variant=0) -> VpDims:

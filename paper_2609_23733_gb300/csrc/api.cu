@@ -425,8 +425,6 @@ vp_status run_layer(const vp_dims* dm, const __nv_bfloat16* xin, const vp_bf16* 
   return VP_OK;
 }
 
-__device__ unsigned int g_linear_err;  // error word of vp_linear (it has no workspace)
-
 }  // namespace
 
 extern "C" {
@@ -583,9 +581,6 @@ vp_status vp_linear(int32_t M, int32_t Nout, int32_t K, const vp_bf16* A, const 
       (bias && !aligned16(bias)) || (scale && !aligned16(scale)))
     return VP_ERR_ALIGNMENT;
   VP_TRY(check_device());
-  unsigned int* err = nullptr;
-  if (cudaGetSymbolAddress(reinterpret_cast<void**>(&err), g_linear_err) != cudaSuccess)
-    return VP_ERR_CUDA;
   LinearArgs la{};
   la.M = M;
   la.N = Nout;
@@ -597,7 +592,6 @@ vp_status vp_linear(int32_t M, int32_t Nout, int32_t K, const vp_bf16* A, const 
   la.scale = scale;
   la.residual = reinterpret_cast<const __nv_bfloat16*>(residual);
   la.out = reinterpret_cast<__nv_bfloat16*>(out);
-  la.err = err;
   return from_cuda(launch_linear(la, device_sm_count(), static_cast<cudaStream_t>(stream)));
 }
 

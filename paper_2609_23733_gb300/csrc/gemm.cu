@@ -98,6 +98,8 @@ __device__ __forceinline__ TileUnit tile_unit(int u, int full_units, int n_tiles
   return r;
 }
 
+__device__ unsigned int g_linear_err;  // error word of calls without a workspace (vp_linear)
+
 // kSkip: the instance that leaves K-blocks out (GemmParams::skip_ids); the other instance has
 // none of that bookkeeping.
 template <bool kSkip, int kEpiWarps, bool kQk = false>
@@ -106,12 +108,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
                 const __grid_constant__ CUtensorMap tmap_b,
                 const __grid_constant__ CUtensorMap tmap_b_cut,
                 const __grid_constant__ CUtensorMap tmap_out,
-                const __grid_constant__ CUtensorMap tmap_res, GemmParams prm) {
+                const __grid_constant__ CUtensorMap tmap_res, const __grid_constant__ GemmParams prm) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   GemmSmem& sm = *reinterpret_cast<GemmSmem*>(smem_raw);
   constexpr int kParts = kEpiWarps / 4;        // column parts of a tile (epilogue warps per lane quarter)
   constexpr int kBufs = kBlocks / kEpiWarps;   // staging blocks of a warp = its 64-column groups
   const int M = prm.M, N = prm.N, K = prm.K;
+  unsigned int* const err = prm.err ? prm.err : &g_linear_err;
   const int n_tiles = (N + kBN - 1) / kBN;
   const int k_blocks = (K + kBK - 1) / kBK;
   const int pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
@@ -142,6 +145,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     tmem_alloc_pair(&sm.tmem_base, kTmemCols);
     tmem_relinquish_pair();
   }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // both CTAs' barriers and TMEM are there
+  tc_fence_after();
   pdl_wait();
   pdl_launch();
   if (kSkip && threadIdx.x == 0) {
@@ -150,10 +157,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     for (int i = s0; i < s1; ++i) mask |= 1u << (prm.skip_ids[i] & 31);
     sm.skip_mask = mask;
   }
-  tc_fence_before();
-  __syncthreads();
-  cluster_sync_all();  // both CTAs' barriers and TMEM are there
-  tc_fence_after();
+  if (kSkip) __syncthreads();
   const uint32_t tmem = __shfl_sync(0xffffffffu, sm.tmem_base, 0);
   // K-blocks left out, and whether that is all of them (A W^T is then 0).
   const uint32_t skip = kSkip ? sm.skip_mask : 0u;
@@ -172,7 +176,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (kSkip && ((skip >> kb) & 1u)) continue;
         const int st = lc % kStages;
-        ok = mbar_wait_warp(&sm.empty[st], ((lc / kStages) & 1) ^ 1, prm.err, abort_flag);
+        ok = mbar_wait_warp(&sm.empty[st], ((lc / kStages) & 1) ^ 1, err, abort_flag);
         if (!ok) break;
         const uint32_t full = cluster_addr(&sm.full[st], 0);
         if (elect_one()) {
@@ -201,7 +205,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     for (int u = pair; rank == 0 && u < prm.units && ok; u += pairs, ++i) {
       const uint32_t idesc = u >= prm.full_units ? id_cut : id_full;
       const uint32_t ab = i & 1;
-      ok = mbar_wait_warp(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1, prm.err, abort_flag);
+      ok = mbar_wait_warp(&sm.acc_empty[ab], ((i >> 1) & 1) ^ 1, err, abort_flag);
       if (!ok) break;
       tc_fence_after();
       const uint32_t d = tmem + ab * kBN;
@@ -209,7 +213,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       for (int kb = 0; kb < k_blocks; ++kb) {
         if (kSkip && ((skip >> kb) & 1u)) continue;
         const int st = lc % kStages;
-        ok = mbar_wait_warp(&sm.full[st], (lc / kStages) & 1, prm.err, abort_flag);
+        ok = mbar_wait_warp(&sm.full[st], (lc / kStages) & 1, err, abort_flag);
         if (!ok) break;
         tc_fence_after();
         const uint64_t da = sdesc_sw128(smem_u32(sm.a[st]));
@@ -314,7 +318,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         for (int b = 0; b < 4; ++b)
           if (2 * b < nb) lnp[b] = lpp[b];
       }
-      const bool ok = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, prm.err, abort_flag);
+      const bool ok = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, err, abort_flag);
       if (!ok) break;
       tc_fence_after();
       // The accumulator goes back to the leader's MMA warp once this warp has read it.
@@ -512,7 +516,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
           if ((cc & 1) == 0) {
             brow = block_begin();
             if (prm.residual &&
-                !mbar_wait_warp(&res_bar[nst % kBufs], (nst / kBufs) & 1, prm.err, abort_flag))
+                !mbar_wait_warp(&res_bar[nst % kBufs], (nst / kBufs) & 1, err, abort_flag))
               break;
           }
           // Bias, GELU, LayerScale and residual on column pairs (packed f32x2 arithmetic).
@@ -644,8 +648,6 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   e = make_tmap_bf16_2d(&tb, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kBN / 2);
   if (e != cudaSuccess) return e;
-  e = make_tmap_bf16_2d(&tb_cut, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kTailN / 2);
-  if (e != cudaSuccess) return e;
   e = make_tmap_bf16_2d(&to, a.out, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N, 64, 32);
   if (e != cudaSuccess) return e;
   tr = to;
@@ -672,6 +674,11 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
   const int left = tiles % pairs_max;
   const int full_units = 2 * left <= pairs_max ? tiles - left : tiles;
   const int units = full_units + 2 * (tiles - full_units);
+  tb_cut = tb;
+  if (full_units < tiles) {
+    e = make_tmap_bf16_2d(&tb_cut, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kTailN / 2);
+    if (e != cudaSuccess) return e;
+  }
   GemmParams prm{a.M,     a.N,   a.K,   a.bias,      a.act,  a.scale,   a.residual,
                  a.out,   a.err, a.ln_part, a.ln_c, a.ln_eps, a.part_out,
                  qk ? a.qk_cols : 0, a.qn_g, a.qn_b, a.kn_g, a.kn_b, a.qk_eps, a.rope_cs,

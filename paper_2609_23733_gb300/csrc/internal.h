@@ -169,7 +169,7 @@ struct LinearArgs {
   const float* scale;
   const __nv_bfloat16* residual;
   __nv_bfloat16* out;
-  unsigned int* err;   // may be NULL (vp_linear has no workspace): a private word is used
+  unsigned int* err;   // NULL (vp_linear has no workspace): a word of the library's own
   // LayerNorm folded into the projection (A is the un-normalised residual stream): with
   // W' = W diag(gamma), c = W' 1 and bias' = b + W beta prepared by launch_ln_fold_weights,
   //   LN(A) W^T + b = rstd_r (A W'^T - mu_r c^T) + bias',
