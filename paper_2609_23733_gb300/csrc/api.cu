@@ -802,6 +802,7 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
     f1.act = VP_ACT_GELU;
     f1.out = hid;
     f1.err = sc.err;
+    f1.w_ready = true;
     VP_TRY(from_cuda(launch_linear(f1, sms, st)));
     LinearArgs f2{};
     f2.M = dims->N;
@@ -816,6 +817,7 @@ vp_status vp_global_stack(const vp_dims* dims, int32_t n_layers, vp_bf16* x_inou
     f2.out = x;
     f2.err = sc.err;
     f2.part_out = part;  // the next block's LN1 statistics
+    f2.w_ready = true;
     VP_TRY(from_cuda(launch_linear(f2, sms, st)));
   }
   return VP_OK;

@@ -33,18 +33,23 @@ namespace vp {
 
 namespace {
 
-constexpr int kBM = 256, kBN = 256, kBK = 64, kStages = 5;  // the pair's tile
-constexpr int kTailN = 128;                                 // width of a cut tile
-constexpr int kABytes = kBM / 2 * kBK * 2;                  // 16 KB: a CTA's half of A
-constexpr uint32_t kTmemCols = 512;
-constexpr int kBlocks = 16;             // staging blocks, shared out over the epilogue warps
-constexpr int kBlkBytes = 32 * 64 * 2;  // a staging block: 32 rows x 64 columns
+constexpr int kBM = 256, kBK = 64;          // rows of the pair's tile, columns of a K block
+constexpr int kTailN = 128;                 // width of a cut tile
+constexpr int kABytes = kBM / 2 * kBK * 2;  // 16 KB: a CTA's half of A
+constexpr int kBlkBytes = 32 * 64 * 2;      // a staging block: 32 rows x 64 columns
 
+// kTileN = 256, or 128 for launches of narrow tiles alone (launch_linear): a stage is then 24 KB, and
+// seven of them cover the copies' latency, which five 32-KB ones with half of B unused did not.
+template <int kTileN>
 struct GemmSmem {
+  static constexpr int kStages = kTileN == 256 ? 5 : 7;
+  static constexpr int kBlocks = kTileN / 16;  // staging blocks, shared out over the epilogue warps
+  static constexpr uint32_t kTmemCols = 2 * kTileN;
   __nv_bfloat16 a[kStages][kBM / 2 * kBK];
-  __nv_bfloat16 b[kStages][kBN / 2 * kBK];
+  __nv_bfloat16 b[kStages][kTileN / 2 * kBK];
   __nv_bfloat16 stage[kBlocks][32 * 64];
-  float vec[2][kBN];        // the tile's bias, and its LayerScale or LN-fold column sums
+  float vec[2][kTileN];     // the tile's bias, and its LayerScale or LN-fold column sums
+  float4 stats[kTileN == 256 ? 1 : 128];  // half a 128-column block's row statistics (part_out)
   uint64_t full[kStages];   // leader's: both CTAs' copies of a stage have landed
   uint64_t empty[kStages];
   uint64_t acc_full[2];
@@ -55,7 +60,7 @@ struct GemmSmem {
   uint32_t skip_mask;  // K-blocks left out (LinearArgs::skip_ids)
   int abort_flag;
 };
-static_assert(sizeof(GemmSmem) <= 232448, "shared memory");
+static_assert(sizeof(GemmSmem<256>) <= 232448 && sizeof(GemmSmem<128>) <= 232448, "shared memory");
 
 struct GemmParams {
   int M, N, K;
@@ -80,6 +85,7 @@ struct GemmParams {
   const int32_t* tok_index;
   const int32_t* skip_ids;
   const int32_t* skip_off;
+  int w_ready;  // LinearArgs::w_ready
   int full_units, units;  // units 0 .. full_units - 1 are whole tiles, the rest halves of tiles
 };
 
@@ -87,6 +93,7 @@ struct GemmParams {
 struct TileUnit {
   int m0, n0, w;
 };
+template <int kBN>
 __device__ __forceinline__ TileUnit tile_unit(int u, int full_units, int n_tiles) {
   const bool cut = u >= full_units;
   const int t = cut ? full_units + ((u - full_units) >> 1) : u;
@@ -102,7 +109,7 @@ __device__ unsigned int g_linear_err;  // error word of calls without a workspac
 
 // kSkip: the instance that leaves K-blocks out (GemmParams::skip_ids); the other instance has
 // none of that bookkeeping.
-template <bool kSkip, int kEpiWarps, bool kQk = false>
+template <bool kSkip, int kEpiWarps, bool kQk = false, int kBN = 256>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps, 1)
     gemm_kernel(const __grid_constant__ CUtensorMap tmap_a,
                 const __grid_constant__ CUtensorMap tmap_b,
@@ -110,7 +117,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
                 const __grid_constant__ CUtensorMap tmap_out,
                 const __grid_constant__ CUtensorMap tmap_res, const __grid_constant__ GemmParams prm) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  GemmSmem& sm = *reinterpret_cast<GemmSmem*>(smem_raw);
+  using Smem = GemmSmem<kBN>;
+  Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  constexpr int kStages = Smem::kStages, kBlocks = Smem::kBlocks;
+  constexpr uint32_t kTmemCols = Smem::kTmemCols;
   constexpr int kParts = kEpiWarps / 4;        // column parts of a tile (epilogue warps per lane quarter)
   constexpr int kBufs = kBlocks / kEpiWarps;   // staging blocks of a warp = its 64-column groups
   const int M = prm.M, N = prm.N, K = prm.K;
@@ -149,6 +159,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
   __syncthreads();
   cluster_sync_all();  // both CTAs' barriers and TMEM are there
   tc_fence_after();
+  // A weight that no kernel just before writes: the first stages' halves of B while that kernel
+  // still runs.
+  int early = 0;  // K blocks of the first unit whose B is on its way
+  if (!kSkip && warp == 0 && prm.w_ready && pair < prm.units) {
+    const TileUnit t = tile_unit<kBN>(pair, prm.full_units, n_tiles);
+    early = min(kStages, k_blocks);
+    for (int kb = 0; kb < early; ++kb) {
+      const uint32_t full = cluster_addr(&sm.full[kb], 0);
+      if (elect_one()) {
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[kb], 2 * (kABytes + t.w / 2 * kBK * 2));
+        tma_load_2d_pair(sm.b[kb], t.w != kBN ? &tmap_b_cut : &tmap_b, full, kb * kBK, t.n0 + rank * (t.w / 2));
+      }
+      __syncwarp();
+    }
+  }
   pdl_wait();
   pdl_launch();
   if (kSkip && threadIdx.x == 0) {
@@ -169,7 +194,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     uint32_t lc = 0;
     bool ok = true;
     for (int u = pair; u < prm.units && ok; u += pairs) {
-      const TileUnit t = tile_unit(u, prm.full_units, n_tiles);
+      const TileUnit t = tile_unit<kBN>(u, prm.full_units, n_tiles);
       const bool cut = t.w != kBN;
       const int row_a = t.m0 + rank * (kBM / 2), row_b = t.n0 + rank * (t.w / 2);
       const uint32_t bytes = 2 * (kABytes + t.w / 2 * kBK * 2);
@@ -179,10 +204,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         ok = mbar_wait_warp(&sm.empty[st], ((lc / kStages) & 1) ^ 1, err, abort_flag);
         if (!ok) break;
         const uint32_t full = cluster_addr(&sm.full[st], 0);
+        const bool b_sent = u == pair && kb < early;
         if (elect_one()) {
-          if (rank == 0) mbar_arrive_expect_tx(&sm.full[st], bytes);
+          if (rank == 0 && !b_sent) mbar_arrive_expect_tx(&sm.full[st], bytes);
           tma_load_2d_pair(sm.a[st], &tmap_a, full, kb * kBK, row_a);
-          tma_load_2d_pair(sm.b[st], cut ? &tmap_b_cut : &tmap_b, full, kb * kBK, row_b);
+          if (!b_sent) tma_load_2d_pair(sm.b[st], cut ? &tmap_b_cut : &tmap_b, full, kb * kBK, row_b);
         }
         __syncwarp();
         ++lc;
@@ -248,6 +274,21 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     uint64_t* res_bar = &sm.res_full[e * kBufs];
     const uint32_t acc_empty0 = cluster_addr(&sm.acc_empty[0], 0);
     auto epi_sync = []() { asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory"); };
+    // The same barrier, and whether p held on every epilogue thread: the warps leave the loop
+    // together when a wait of one of them gave up, so that none is left at a barrier.
+    auto epi_all = [](bool p) -> bool {
+      uint32_t r;
+      asm volatile(
+          "{\n\t.reg .pred pi, po;\n\t"
+          "setp.ne.u32 pi, %1, 0;\n\t"
+          "bar.red.and.pred po, 1, %2, pi;\n\t"
+          "selp.u32 %0, 1, 0, po;\n\t}"
+          : "=r"(r)
+          : "r"((uint32_t)p), "n"(32 * kEpiWarps)
+          : "memory");
+      return r != 0;
+    };
+    bool alive = true;
     if (acc_zero) {
       // Every K-block is left out, so no MMA writes the accumulators: zero this thread's
       // columns of both once, and every tile then reads A W^T = 0.
@@ -255,7 +296,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
 #pragma unroll
       for (int k = 0; k < 32; ++k) z[k] = 0.f;
 #pragma unroll
-      for (int q = 0; q < 16 / kParts; ++q) tmem_st32(t_lane + (part * (16 / kParts) + q) * 32, z);
+      for (int q = 0; q < kBN / 16 / kParts; ++q) tmem_st32(t_lane + (part * (kBN / 16 / kParts) + q) * 32, z);
       tmem_wait_st();
       // a cut tile's columns are read by other warps of the lane quarter than zeroed them
       tc_fence_before();
@@ -264,7 +305,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     }
     uint32_t i = 0, nst = 0;
     for (int u = pair; u < prm.units; u += pairs, ++i) {
-      const TileUnit t = tile_unit(u, prm.full_units, n_tiles);
+      const TileUnit t = tile_unit<kBN>(u, prm.full_units, n_tiles);
       const uint32_t ab = i & 1;
       // This warp's columns of the tile: n_grp groups of 64 from pcol0.  A cut tile's two groups
       // go to the first two parts, or both to the first one where a thread needs a whole
@@ -299,7 +340,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         const float* second = prm.scale ? prm.scale : prm.ln_c;
         const float v0 = in && prm.bias ? prm.bias[col] : 0.f;
         const float v1 = in && second ? second[col] : 0.f;
-        epi_sync();  // every warp is done with the previous tile's
+        if (!epi_all(alive)) break;  // every warp is done with the previous tile's
         if (et < kBN) {
           sm.vec[0][et] = v0;
           sm.vec[1][et] = v1;
@@ -318,8 +359,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         for (int b = 0; b < 4; ++b)
           if (2 * b < nb) lnp[b] = lpp[b];
       }
-      const bool ok = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, err, abort_flag);
-      if (!ok) break;
+      alive = mbar_wait_warp(&sm.acc_full[ab], (i >> 1) & 1, err, abort_flag);
+      if (!alive) {
+        if (kBN == 128 && prm.part_out) asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
+        continue;
+      }
       tc_fence_after();
       // The accumulator goes back to the leader's MMA warp once this warp has read it.
       auto release_acc = [&]() {
@@ -356,7 +400,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         }
         ln_rstd = rsqrtf(m2 / (float)K + prm.ln_eps);
       }
-      float cmean[4], cm2[4];  // output statistics per 32-column chunk (part_out)
+      float cmean[4] = {}, cm2[4] = {};  // output statistics per 32-column chunk (part_out)
       const uint32_t tcol = t_lane + ab * kBN + (pcol0 - t.n0);
       // Bias, or the folded LayerNorm rstd (acc - mu c) + bias', on one 32-column chunk.
       auto bias_fold = [&](float* x, int col0) {
@@ -516,8 +560,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
           if ((cc & 1) == 0) {
             brow = block_begin();
             if (prm.residual &&
-                !mbar_wait_warp(&res_bar[nst % kBufs], (nst / kBufs) & 1, err, abort_flag))
+                !mbar_wait_warp(&res_bar[nst % kBufs], (nst / kBufs) & 1, err, abort_flag)) {
+              alive = false;
               break;
+            }
           }
           // Bias, GELU, LayerScale and residual on column pairs (packed f32x2 arithmetic).
           bias_fold(x, col0);
@@ -575,13 +621,27 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         tmem_wait_ld();
         if (cc + 2 == 2 * n_grp) release_acc();  // the last chunk is in registers
       }
-      const int pcol = pcol0;  // this thread's 128-column block
-      if (!kQk && kParts == 2 && prm.part_out && row_ok && pcol < N) {
-        const float mb = 0.25f * (cmean[0] + cmean[1] + cmean[2] + cmean[3]);
-        float m2 = cm2[0] + cm2[1] + cm2[2] + cm2[3];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) m2 += 32.f * (cmean[k] - mb) * (cmean[k] - mb);
-        prm.part_out[(size_t)row * (N >> 7) + (pcol >> 7)] = make_float2(mb, m2);
+      if (!kQk && kParts == 2 && prm.part_out) {  // this row's (mean, M2) of a 128-column block
+        float c2 = cmean[2], c3 = cmean[3], q2 = cm2[2], q3 = cm2[3];
+        if (kBN == 128) {  // the block's second half is the other warp's of this lane quarter
+          float4* st4 = &sm.stats[quarter * 32 + lane];
+          if (part == 1) *st4 = make_float4(cmean[0], cmean[1], cm2[0], cm2[1]);
+          asm volatile("bar.sync %0, 64;" ::"r"(2 + quarter) : "memory");
+          const float4 o = *st4;
+          c2 = o.x;
+          c3 = o.y;
+          q2 = o.z;
+          q3 = o.w;
+        }
+        if (row_ok && pcol0 < N && (kBN == 256 || part == 0)) {
+          const float mb = 0.25f * (cmean[0] + cmean[1] + c2 + c3);
+          float m2 = cm2[0] + cm2[1] + q2 + q3;
+          m2 += 32.f * (cmean[0] - mb) * (cmean[0] - mb);
+          m2 += 32.f * (cmean[1] - mb) * (cmean[1] - mb);
+          m2 += 32.f * (c2 - mb) * (c2 - mb);
+          m2 += 32.f * (c3 - mb) * (c3 - mb);
+          prm.part_out[(size_t)row * (N >> 7) + (pcol0 >> 7)] = make_float2(mb, m2);
+        }
       }
     }
     if (elect_one()) tma_store_wait_read<0>();  // the staging blocks outlive the reads
@@ -646,8 +706,6 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
   CUtensorMap ta, tb, tb_cut, to, tr;
   cudaError_t e = make_tmap_bf16_2d(&ta, a.A, (uint64_t)a.K, (uint64_t)a.M, (uint64_t)a.K, kBK, kBM / 2);
   if (e != cudaSuccess) return e;
-  e = make_tmap_bf16_2d(&tb, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kBN / 2);
-  if (e != cudaSuccess) return e;
   e = make_tmap_bf16_2d(&to, a.out, (uint64_t)a.N, (uint64_t)a.M, (uint64_t)a.N, 64, 32);
   if (e != cudaSuccess) return e;
   tr = to;
@@ -667,15 +725,20 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
     return cudaErrorInvalidValue;
   // Whole rounds of 256 x 256 tiles over the pairs; a last round that at most half of the pairs
   // would work on is cut into tiles of half the width (10,992 x 1,024 from K = 4,096: 172 tiles
-  // on 76 pairs; 1,044 rows: 20 tiles become 40, K = 4,096 28.0 us with 128 x 256 tiles of single
-  // CTAs, 16.5 here).
+  // on 76 pairs).  Where that is all there is, the instance of 128-wide tiles runs (1,044 rows,
+  // K = 4,096: 20 tiles become 40; 28.0 us with 128 x 256 tiles of single CTAs, 16.5 with cut tiles,
+  // 14.4 with this instance).
   const int pairs_max = max(1, num_sms / 2);
-  const int tiles = ((a.M + kBM - 1) / kBM) * ((a.N + kBN - 1) / kBN);
+  const int m_tiles = (a.M + kBM - 1) / kBM;
+  const int tiles = m_tiles * ((a.N + 255) / 256);
   const int left = tiles % pairs_max;
-  const int full_units = 2 * left <= pairs_max ? tiles - left : tiles;
-  const int units = full_units + 2 * (tiles - full_units);
+  const bool narrow = !qk && 2 * tiles <= pairs_max;
+  const int full_units = narrow ? m_tiles * ((a.N + 127) / 128) : 2 * left <= pairs_max ? tiles - left : tiles;
+  const int units = narrow ? full_units : full_units + 2 * (tiles - full_units);
+  e = make_tmap_bf16_2d(&tb, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, narrow ? 64 : 128);
+  if (e != cudaSuccess) return e;
   tb_cut = tb;
-  if (full_units < tiles) {
+  if (full_units < units && !narrow) {
     e = make_tmap_bf16_2d(&tb_cut, a.W, (uint64_t)a.K, (uint64_t)a.N, (uint64_t)a.K, kBK, kTailN / 2);
     if (e != cudaSuccess) return e;
   }
@@ -683,10 +746,10 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
                  a.out,   a.err, a.ln_part, a.ln_c, a.ln_eps, a.part_out,
                  qk ? a.qk_cols : 0, a.qn_g, a.qn_b, a.kn_g, a.kn_b, a.qk_eps, a.rope_cs,
                  a.rope_npos, a.tok_per_view, a.patch_start, a.grid_w, a.tok_index, a.skip_ids, a.skip_off,
-                 full_units, units};
+                 a.w_ready ? 1 : 0, full_units, units};
   const int grid = 2 * min(pairs_max, units);
-  const int smem = (int)sizeof(GemmSmem);
-  auto launch = [&](auto kernel, int epi_warps) -> cudaError_t {
+  auto launch = [&](auto kernel, int epi_warps, size_t smem_bytes = sizeof(GemmSmem<256>)) -> cudaError_t {
+    const int smem = (int)smem_bytes;
     cudaError_t le = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (le != cudaSuccess) return le;
     prof_before(VP_KERNEL_GEMM, st);
@@ -694,6 +757,9 @@ cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st) {
     prof_after(st);
     return le;
   };
+  if (narrow)
+    return a.skip_ids ? launch(gemm_kernel<true, 8, false, 128>, 8, sizeof(GemmSmem<128>))
+                      : launch(gemm_kernel<false, 8, false, 128>, 8, sizeof(GemmSmem<128>));
   // Sixteen epilogue warps (64 columns of a row per thread, one staging block each) where the
   // epilogue is what a tile waits for: GELU (137,400 x 4,096 from K = 1,024: 668 us with eight
   // warps, 655 with sixteen), and a single round, whose epilogue no next tile covers (1,044 x

@@ -197,6 +197,9 @@ struct LinearArgs {
   // 32 x 64; no LayerNorm fold, no qk columns).  NULL: none.
   const int32_t* skip_ids;
   const int32_t* skip_off;
+  // The kernel just before this one in the stream is the library's own and does not write W: its
+  // first tiles may be read before that kernel has completed.
+  bool w_ready;
 };
 cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st);
 
