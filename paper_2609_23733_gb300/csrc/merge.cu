@@ -46,6 +46,8 @@ __device__ __forceinline__ int source_index(const MergeGeo& g, int i) {
 __global__ void metric_weights_kernel(const __nv_bfloat16* w_qkv, const float* b_qkv, int H,
                                       int D, __nv_bfloat16* wbar, float* bbar) {
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_launch();
   if (idx >= 64 * D) return;
   const int c = idx / D, k = idx - c * D;
   float s = 0.f;
@@ -61,11 +63,15 @@ __global__ void metric_weights_kernel(const __nv_bfloat16* w_qkv, const float* b
 
 // Eight lanes per token (16 bytes each, four tokens per warp): the metric row as a unit vector
 // (bf16), stored by source index for a source and by merged row for a destination; the
-// merged row of every token (-1 for sources) and the token of every merged row.
+// merged row of every token (-1 for sources) and the token of every merged row.  Clears what the
+// kernels behind it count and compare in: a source's best key, a merged row's counters.
 __global__ void merge_setup_kernel(MergeGeo g, const __nv_bfloat16* kbar, __nv_bfloat16* m_src,
-                                   __nv_bfloat16* m_dst, int* row_of, int* dst_tok) {
+                                   __nv_bfloat16* m_dst, int* row_of, int* dst_tok,
+                                   unsigned long long* best, int* cnt, int* fill) {
   const int sub = threadIdx.x & 7;
   const int i = blockIdx.x * (blockDim.x >> 3) + (threadIdx.x >> 3);
+  pdl_wait();
+  pdl_launch();
   if (i >= g.N) return;  // whole groups of eight lanes leave together
   const uint4 u = reinterpret_cast<const uint4*>(kbar + (size_t)i * 64)[sub];
   const uint32_t w[4] = {u.x, u.y, u.z, u.w};
@@ -86,7 +92,13 @@ __global__ void merge_setup_kernel(MergeGeo g, const __nv_bfloat16* kbar, __nv_b
   reinterpret_cast<uint4*>(dst)[sub] = make_uint4(mu[0], mu[1], mu[2], mu[3]);
   if (sub == 0) {
     row_of[i] = r;
-    if (r >= 0) dst_tok[r] = i;
+    if (r >= 0) {
+      dst_tok[r] = i;
+      cnt[r] = 0;
+      fill[r] = 0;
+    } else {
+      best[source_index(g, i)] = 0ull;
+    }
   }
 }
 
@@ -165,7 +177,10 @@ __global__ void __launch_bounds__(kMatchThreads, 1)
   const long long n_units = (long long)n_tiles * n_chunks;
   const long long u_begin = n_units * blockIdx.x / gridDim.x;
   const long long u_end = n_units * (blockIdx.x + 1) / gridDim.x;
-  if (u_begin >= u_end) return;  // uniform across the CTA
+  if (u_begin >= u_end) {  // uniform across the CTA
+    pdl_wait();
+    return;
+  }
   const int warp = warp_uniform_id(), lane = lane_id();
   volatile int* abort_flag = &sm.abort_flag;
   if (threadIdx.x == 0) {
@@ -191,6 +206,8 @@ __global__ void __launch_bounds__(kMatchThreads, 1)
     tmem_alloc(&sm.tmem_base, kMatchTmemCols);
     tmem_relinquish();
   }
+  pdl_wait();
+  pdl_launch();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -373,6 +390,8 @@ __global__ void __launch_bounds__(kMatchThreads, 1)
 __global__ void merge_resolve_kernel(MergeGeo g, const int* row_of, const unsigned long long* best,
                                      int* assign, int* cnt) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_launch();
   if (i >= g.N) return;
   int r = row_of[i];
   if (r < 0) {
@@ -400,6 +419,8 @@ __global__ void __launch_bounds__(1024) scan_kernel(int n, const int* cnt, int* 
     if (i + 2 < n) r.z = cnt[i + 2];
     return r;
   };
+  pdl_wait();
+  pdl_launch();
   int carry = 0;
   int4 nxt = load4(0);
   for (int base = 0; base < n; base += 4096) {
@@ -444,6 +465,8 @@ __global__ void __launch_bounds__(1024) scan_kernel(int n, const int* cnt, int* 
 __global__ void merge_fill_kernel(int N, const int* assign, const int* offs, int* fill,
                                   int* members) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_wait();
+  pdl_launch();
   if (i >= N) return;
   const int r = assign[i];
   members[offs[r] + atomicAdd(fill + r, 1)] = i;
@@ -471,10 +494,10 @@ __device__ __forceinline__ void store_mean(const float (&acc)[C][8], float inv, 
 #pragma unroll
   for (int c = 0; c < C; ++c) {
     const int col = (c * 32 + lane) * 8;
-    const float4 g0 = __ldg(reinterpret_cast<const float4*>(gamma + col));
-    const float4 g1 = __ldg(reinterpret_cast<const float4*>(gamma + col) + 1);
-    const float4 b0 = __ldg(reinterpret_cast<const float4*>(beta + col));
-    const float4 b1 = __ldg(reinterpret_cast<const float4*>(beta + col) + 1);
+    const float4 g0 = reinterpret_cast<const float4*>(gamma + col)[0];
+    const float4 g1 = reinterpret_cast<const float4*>(gamma + col)[1];
+    const float4 b0 = reinterpret_cast<const float4*>(beta + col)[0];
+    const float4 b1 = reinterpret_cast<const float4*>(beta + col)[1];
     const float gg[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
     const float bb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
     uint4 o;
@@ -495,7 +518,7 @@ __device__ __forceinline__ void flush_row(float (&acc)[C][8], int r, int a, int 
                                           float* slots, const float* gamma, const float* beta,
                                           __nv_bfloat16* xm) {
   constexpr int D = 256 * C;
-  const int first = __ldg(offs + r), last = __ldg(offs + r + 1);
+  const int first = offs[r], last = offs[r + 1];
   if (first < q0 || last > q0 + nm) {  // the row crosses a chunk boundary
     float* slot = slots + ((size_t)ch * 2 + (first < q0 ? 0 : 1)) * D;
 #pragma unroll
@@ -547,10 +570,46 @@ __global__ void __launch_bounds__(256, C <= 2 ? 3 : (C <= 4 ? 2 : 1))
   const int lane = threadIdx.x & 31;
   const int ch = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int q0 = ch * kMeanChunk;
+  pdl_wait();
+  pdl_launch();
   if (q0 >= N) return;
   const int nm = min(kMeanChunk, N - q0);
-  const int mine = lane < nm ? __ldg(members + q0 + lane) : 0;  // one coalesced load
-  const int my_row = lane < nm ? __ldg(assign + mine) : -1;
+  const int mine = lane < nm ? members[q0 + lane] : 0;  // one coalesced load
+  const int my_row = lane < nm ? assign[mine] : -1;
+  // Lane l: mean and 1 / sqrt(var + eps) of member l's row from its 128-column blocks, summed as a
+  // tree: per row over the lanes, ten shuffles one after another set the time (137,400 tokens to
+  // 15,432 rows: 82 -> 70 us).
+  float my_rstd, my_nmr;
+  {
+    constexpr int NP = NB <= 2 ? 2 : NB <= 4 ? 4 : NB <= 8 ? 8 : NB <= 16 ? 16 : 32;
+    float bm[NP], bq[NP];
+    const float2* ps = part + (size_t)mine * NB;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const float2 v = k < NB ? ps[k] : make_float2(0.f, 0.f);
+      bm[k] = v.x;
+      bq[k] = v.y;
+    }
+    float t[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) t[k] = bm[k];
+#pragma unroll
+    for (int o = NP / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) t[k] += t[k + o];
+    const float mu = t[0] / (float)NB;
+#pragma unroll
+    for (int k = 0; k < NP; ++k) {
+      const float d = bm[k] - mu;
+      t[k] = k < NB ? bq[k] + 128.f * d * d : 0.f;
+    }
+#pragma unroll
+    for (int o = NP / 2; o > 0; o >>= 1)
+#pragma unroll
+      for (int k = 0; k < o; ++k) t[k] += t[k + o];
+    my_rstd = rsqrtf(t[0] / (float)D + eps);
+    my_nmr = -mu * my_rstd;
+  }
   float acc[C][8];
 #pragma unroll
   for (int c = 0; c < C; ++c)
@@ -560,14 +619,12 @@ __global__ void __launch_bounds__(256, C <= 2 ? 3 : (C <= 4 ? 2 : 1))
   // Entries 0 .. nm - 1, then a sentinel entry nm that ends the last row (one flush site).
   for (int k = 0; k <= nm; k += kMeanInFlight) {  // the rows' loads issued before any arithmetic
     uint4 u[kMeanInFlight][C];
-    float2 ps[kMeanInFlight];
 #pragma unroll
     for (int j = 0; j < kMeanInFlight; ++j) {
       const int i = __shfl_sync(0xffffffffu, mine, min(k + j, nm - 1));
 #pragma unroll
       for (int c = 0; c < C; ++c)
-        u[j][c] = __ldg(reinterpret_cast<const uint4*>(x + (size_t)i * D + (c * 32 + lane) * 8));
-      ps[j] = lane < NB ? __ldg(part + (size_t)i * NB + lane) : make_float2(0.f, 0.f);
+        u[j][c] = *reinterpret_cast<const uint4*>(x + (size_t)i * D + (c * 32 + lane) * 8);
     }
 #pragma unroll
     for (int j = 0; j < kMeanInFlight; ++j) {
@@ -585,16 +642,7 @@ __global__ void __launch_bounds__(256, C <= 2 ? 3 : (C <= 4 ? 2 : 1))
         run0 = e;
       }
       if (e == nm) break;
-      float sm = ps[j].x;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, o);
-      const float mu = sm / (float)NB;
-      const float d = ps[j].x - mu;
-      float m2 = lane < NB ? ps[j].y + 128.f * d * d : 0.f;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-      const float rstd = rsqrtf(m2 / (float)D + eps);
-      const float nmr = -mu * rstd;
+      const float rstd = __shfl_sync(0xffffffffu, my_rstd, e), nmr = __shfl_sync(0xffffffffu, my_nmr, e);
 #pragma unroll
       for (int c = 0; c < C; ++c) {
         const uint32_t w[4] = {u[j][c].x, u[j][c].y, u[j][c].z, u[j][c].w};
@@ -612,6 +660,8 @@ __global__ void __launch_bounds__(256, C <= 2 ? 3 : (C <= 4 ? 2 : 1))
 // x[i] <- bf16(x[i] + ls (.) a[assign[i]]) (unmerge, LayerScale, residual add) and
 // z[i] = LN(x[i]) (gamma, beta, eps) from the stored bf16 values, in one pass over the rows
 // (the LayerNorm kernel's arithmetic: fp32 mean, then the biased variance about it).
+// Launched the ordinary way, with read-only loads: behind a griddepcontrol.wait, with plain loads, it
+// took 178 us instead of 159.
 template <int C>
 __global__ void __launch_bounds__(256, 4) unmerge_ln_kernel(int N, const int* assign,
                                                             const __nv_bfloat16* a, const float* ls,
@@ -704,9 +754,9 @@ cudaError_t launch_merge_prepare(const MergeGeo& g, int H, const __nv_bfloat16* 
                                  cudaStream_t st) {
   const int D = 64 * H;
   prof_before(VP_KERNEL_MERGE, st);
-  metric_weights_kernel<<<(64 * D + 255) / 256, 256, 0, st>>>(w_qkv, b_qkv, H, D, s.wbar, s.bbar);
+  cudaError_t e = launch_pdl(metric_weights_kernel, dim3((64 * D + 255) / 256), 256, 0, st, w_qkv, b_qkv, H,
+                             D, s.wbar, s.bbar);
   prof_after(st);
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // The metric of LN1(x) with LN1 folded into its weights, as in the QKV projection.
   if ((e = launch_ln_fold_weights(64, D, s.wbar, ln.g, ln.b, s.bbar, ln.w_fold, ln.c_fold,
@@ -728,10 +778,9 @@ cudaError_t launch_merge_prepare(const MergeGeo& g, int H, const __nv_bfloat16* 
   e = launch_linear(la, num_sms, st);
   if (e != cudaSuccess) return e;
   prof_before(VP_KERNEL_MERGE, st);
-  merge_setup_kernel<<<(g.N + 31) / 32, 256, 0, st>>>(g, s.kbar, s.m_src, s.m_dst, s.row_of,
-                                                      s.dst_tok);
+  e = launch_pdl(merge_setup_kernel, dim3((g.N + 31) / 32), 256, 0, st, g, s.kbar, s.m_src, s.m_dst,
+                 s.row_of, s.dst_tok, s.best, s.cnt, s.fill);
   prof_after(st);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (g.Ns > 0) {  // one view, or stride 1: every token is a destination
     CUtensorMap tsrc, tdst;  // unit metric rows, 64 channels (128 bytes), 128-byte swizzle
@@ -746,31 +795,26 @@ cudaError_t launch_merge_prepare(const MergeGeo& g, int H, const __nv_bfloat16* 
     const long long units =
         (long long)((g.Ns + 127) / 128) * ((g.Np + kMatchN - 1) / kMatchN);
     prof_before(VP_KERNEL_MERGE, st);
-    e = cudaMemsetAsync(s.best, 0, (size_t)g.Ns * sizeof(unsigned long long), st);
-    if (e == cudaSuccess) {
-      tome_match_kernel<<<(int)min((long long)num_sms, units), kMatchThreads, smem, st>>>(
-          tsrc, tdst, g, s.best, s.err);
-      e = cudaGetLastError();
-    }
+    e = launch_pdl(tome_match_kernel, dim3((int)min((long long)num_sms, units)), kMatchThreads, smem, st,
+                   tsrc, tdst, g, s.best, s.err);
     prof_after(st);
     if (e != cudaSuccess) return e;
   }
-  if ((e = cudaMemsetAsync(s.cnt, 0, (size_t)g.Np * sizeof(int), st)) != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(s.fill, 0, (size_t)g.Np * sizeof(int), st)) != cudaSuccess) return e;
   prof_before(VP_KERNEL_MERGE, st);
-  merge_resolve_kernel<<<(g.N + 255) / 256, 256, 0, st>>>(g, s.row_of, s.best, s.assign, s.cnt);
-  scan_kernel<<<1, 1024, 0, st>>>(g.Np, s.cnt, s.offs);
-  merge_fill_kernel<<<(g.N + 255) / 256, 256, 0, st>>>(g.N, s.assign, s.offs, s.fill, s.members);
+  e = launch_pdl(merge_resolve_kernel, dim3((g.N + 255) / 256), 256, 0, st, g, s.row_of, s.best, s.assign, s.cnt);
+  if (e == cudaSuccess) e = launch_pdl(scan_kernel, dim3(1), 1024, 0, st, g.Np, s.cnt, s.offs);
+  if (e == cudaSuccess)
+    e = launch_pdl(merge_fill_kernel, dim3((g.N + 255) / 256), 256, 0, st, g.N, s.assign, s.offs, s.fill,
+                   s.members);
   prof_extra_launch();
   prof_extra_launch();
   prof_after(st);
-  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   prof_before(VP_KERNEL_MERGE, st);
   const int grid = ((g.N + kMeanChunk - 1) / kMeanChunk + 7) / 8;  // a warp per chunk
 #define VP_MEAN(C_)                                                                              \
-  merge_mean_kernel<C_><<<grid, 256, 0, st>>>(g.N, x, ln.part, ln.g, ln.b, ln.eps, s.offs,       \
-                                              s.members, s.assign, s.fill, s.slots, s.xm)
+  e = launch_pdl(merge_mean_kernel<C_>, dim3(grid), 256, 0, st, g.N, x, ln.part, ln.g, ln.b,     \
+                 ln.eps, s.offs, s.members, s.assign, s.fill, s.slots, s.xm)
   switch (D / 256) {
     case 1: VP_MEAN(1); break;
     case 2: VP_MEAN(2); break;
@@ -781,7 +825,7 @@ cudaError_t launch_merge_prepare(const MergeGeo& g, int H, const __nv_bfloat16* 
     default: prof_after(st); return cudaErrorInvalidValue;
   }
   prof_after(st);
-  return cudaGetLastError();
+  return e;
 }
 
 cudaError_t launch_unmerge_ln(int N, int D, const int* assign, const __nv_bfloat16* a,
