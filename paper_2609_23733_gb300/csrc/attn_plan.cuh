@@ -32,16 +32,18 @@ struct Plan {
 // From kShortTiles key tiles on, S minimises the last round's length in key tiles,
 //   ceil(T S / P) (n_kv / S + kUnitTiles) + kCombineTiles S   (S = 1: no combine).
 // kUnitTiles, the cost of a unit beyond its keys (Q load, pipeline fill and drain, partial store),
-// and kCombineTiles, what a part adds to the combine, are fitted to a sweep of S at 10,992
-// tokens; being costs in time they do not shrink with n_kv.
+// and kCombineTiles, what a part adds to the combine, are fitted to sweeps at 1 to 16 heads and
+// 2,748 to 137,400 tokens; being costs in time they do not shrink with n_kv.  (13 and 1.5, which fitted
+// while a group's last part combined it, took 1.1 % longer in the mean of 17 shapes: 3 heads at
+// 10,992 tokens 116.7 us against 111.8, 1 at 15,432 84.0 against 79.7, at 43,968 435 against 432.)
 // Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
-// 10,992 tokens 466 -> 394 us (8 groups left over: 19 parts -> 11), 3 heads 166 -> 119, 1 head at
-// 15,432 tokens 101 -> 92.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
+// 10,992 tokens 466 -> 383 us (8 groups left over: 19 parts -> 13), 3 heads 166 -> 112, 1 head at
+// 15,432 tokens 101 -> 80.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
 // 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
 // there: a deep stack of short sequences then gives the same bits as it always did.
 constexpr int kMaxParts = 64;
 constexpr int kMaxTailUnits = kFaTailUnits * 4 / kFaChains;  // the scratch is sized for four chains
-constexpr float kUnitTiles = 13.f, kCombineTiles = 1.5f;
+constexpr float kUnitTiles = 7.f, kCombineTiles = 1.f;
 constexpr int kShortTiles = 41;
 constexpr float kPartShare = 0.03f;
 
