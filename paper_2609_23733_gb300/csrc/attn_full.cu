@@ -173,7 +173,7 @@ __device__ __noinline__ void split_part(FullParams prm, int part_slot, int c, in
 }
 
 // kParts = false: the whole groups (all of them when nothing is split); kParts = true: the
-// split parts, one per CTA, launched right behind (programmatic dependent launch) so that
+// split parts, handed out by a counter, launched right behind (programmatic dependent launch) so that
 // they take the SMs the whole groups leave.  Two instantiations keep runtime key ranges out
 // of the main one's attention loop, which they would slow down by about a tenth.
 template <bool kParts>

@@ -4,20 +4,11 @@
 
 #include <math.h>
 
+#include "attn_split.h"
 #include "common.cuh"
 #include "internal.h"
 
 namespace vp {
-
-#ifndef VP_ATTN_CHAINS
-#define VP_ATTN_CHAINS 3
-#endif
-#ifndef VP_ATTN_BN
-#define VP_ATTN_BN 64
-#endif
-constexpr int kFaChains = VP_ATTN_CHAINS;  // query tiles (chains) of a group
-constexpr int kFaRows = 128;               // query rows of a tile
-constexpr int kFaKeys = VP_ATTN_BN;        // keys of a tile
 
 struct Plan {
   int R, T, S, units;
@@ -28,25 +19,8 @@ struct Plan {
 // first R = floor(G / P) rounds take whole groups; the T = G - R P groups of the last round
 // are split along the keys into S parts each (at most the number of key tiles), T S part units,
 // so the last round lasts about ceil(T S / P) parts of a group instead of one whole group on T
-// CTAs.  Unit u < R P is group u; unit R P + S t + s is part s of group R P + t.
-// From kShortTiles key tiles on, S minimises the last round's length in key tiles,
-//   ceil(T S / P) (n_kv / S + kUnitTiles) + kCombineTiles S   (S = 1: no combine).
-// kUnitTiles, the cost of a unit beyond its keys (Q load, pipeline fill and drain, partial store),
-// and kCombineTiles, what a part adds to the combine, are fitted to sweeps at 1 to 16 heads and
-// 2,748 to 137,400 tokens; being costs in time they do not shrink with n_kv.  (13 and 1.5, which fitted
-// while a group's last part combined it, took 1.1 % longer in the mean of 17 shapes: 3 heads at
-// 10,992 tokens 116.7 us against 111.8, 1 at 15,432 84.0 against 79.7, at 43,968 435 against 432.)
-// Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
-// 10,992 tokens 466 -> 383 us (8 groups left over: 19 parts -> 13), 3 heads 166 -> 112, 1 head at
-// 15,432 tokens 101 -> 80.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
-// 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
-// there: a deep stack of short sequences then gives the same bits as it always did.
-constexpr int kMaxParts = 64;
-constexpr int kMaxTailUnits = kFaTailUnits * 4 / kFaChains;  // the scratch is sized for four chains
-constexpr float kUnitTiles = 7.f, kCombineTiles = 1.f;
-constexpr int kShortTiles = 41;
-constexpr float kPartShare = 0.03f;
-
+// CTAs.  Unit u < R P is group u; unit R P + S t + s is part s of group R P + t.  attn_split.h chooses S.
+//
 // Called by whole warps: lane l weighs S = l + 1 and l + 33 (a loop over S in every thread took
 // several microseconds of every launch).
 __device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_only) {
@@ -56,32 +30,12 @@ __device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_onl
   pl.T = G - pl.R * P;
   pl.S = 1;
   if (pl.T > 0) {
-    float best = INFINITY;
-    int bs = 1;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const int S = lane_id() + 1 + 32 * k;
-      const bool brief = n_kv < kShortTiles;
-      if (S > 1 && (S > n_kv || pl.T * S > (brief ? kFaTailUnits : kMaxTailUnits))) continue;
-      const float rounds = (float)((pl.T * S + P - 1) / P);
-      const float cost = brief ? (S == 1 ? 1.f : rounds * (1.f / (float)S + kPartShare))
-                               : rounds * ((float)n_kv / (float)S + kUnitTiles) +
-                                     (S > 1 ? kCombineTiles * (float)S : 0.f);
-      if (cost < best) {
-        best = cost;
-        bs = S;
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {  // smallest cost, then smallest S: the same on every lane
-      const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int os = __shfl_xor_sync(0xffffffffu, bs, o);
-      if (ob < best || (ob == best && os < bs)) {
-        best = ob;
-        bs = os;
-      }
-    }
-    pl.S = bs;
+    const int s0 = lane_id() + 1, s1 = s0 + 32;
+    const uint32_t c0 = split_allowed(pl.T, n_kv, s0) ? split_cost(pl.T, P, n_kv, s0) : 0xffffffffu;
+    const uint32_t c1 = split_allowed(pl.T, n_kv, s1) ? split_cost(pl.T, P, n_kv, s1) : 0xffffffffu;
+    const uint32_t best = __reduce_min_sync(0xffffffffu, min(c0, c1));
+    const uint32_t lo = __ballot_sync(0xffffffffu, c0 == best), hi = __ballot_sync(0xffffffffu, c1 == best);
+    pl.S = lo ? __ffs(lo) : 32 + __ffs(hi);
   }
   pl.units = pl.S == 1 ? G : pl.R * P + pl.T * pl.S;
   pl.whole = parts_only ? 0 : (pl.S == 1 ? G : pl.R * P);

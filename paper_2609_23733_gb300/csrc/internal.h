@@ -9,6 +9,7 @@
 
 #include <utility>
 
+#include "attn_split.h"
 #include "vp.h"
 
 namespace vp {
@@ -45,8 +46,7 @@ struct RouterScratch {
 
 // Full attention splits the work items of its last, partial round along the keys over the
 // CTAs that would otherwise idle; the partial results need this much scratch (units = groups
-// x splits of that round, at most one per CTA).
-constexpr int kFaTailUnits = 512;
+// x parts of that round, at most kMaxTailUnits).
 constexpr size_t kFaPartFloats = (size_t)kFaTailUnits * 4 * 128 * 64;
 constexpr size_t kFaStatsFloats = (size_t)kFaTailUnits * 4 * 128 * 4;
 // Counters of the head modes: split parts, cheap-head items and columns of W_O's bias handed out.
