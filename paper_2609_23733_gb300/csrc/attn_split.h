@@ -6,11 +6,7 @@
 
 #include <stdint.h>
 
-#ifdef __CUDACC__
-#define VP_HOST_DEVICE __host__ __device__ __forceinline__
-#else
-#define VP_HOST_DEVICE inline
-#endif
+#include "host_device.h"
 
 namespace vp {
 

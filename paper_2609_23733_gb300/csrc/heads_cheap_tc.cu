@@ -45,6 +45,7 @@
 // waits (bounded) for its own copies and MMAs, frees TMEM and exits.
 #include "attn_plan.cuh"
 #include "common.cuh"
+#include "heads_vec.h"
 #include "internal.h"
 
 namespace vp {
@@ -58,6 +59,7 @@ constexpr int kTcGroups = 2;      // epilogue groups (= TMEM accumulators)
 constexpr int kTcBatch = 4;       // items taken from the counter at a time (one when there are few)
 constexpr int kTcParts = 2;       // epilogue warps per TMEM lane quarter in a group
 constexpr int kGroupThreads = 128 * kTcParts;
+static_assert(2 * kTcGroups <= kMaxHeads, "vec_entry");
 constexpr int kTcThreads = 64 + kGroupThreads * kTcGroups;
 // A row's work split over the kTcParts warps of its lane quarter: part p takes the chunk
 // range [begin(p), begin(p + 1)) of the n chunks, as even as possible.  The first layer's
@@ -76,7 +78,8 @@ struct TcSmem {
   __nv_bfloat16 w1[2][128 * 64];
   __nv_bfloat16 w2[2][128 * 64];
   __nv_bfloat16 ys[4 * kTcParts * kTcGroups][32 * 32];  // a warp's output block, 64-byte swizzle
-  // Every surrogate head's vectors, by slot in the surrogate bin, computed at kernel start:
+  // Surrogate heads' vectors: every head's by slot in the surrogate bin, computed at kernel start, or with
+  // single items two entries per epilogue group (vec_entry), computed when a tile first needs them:
   // W1[:, d:] C_h + b1 (gamma | delta), -log2(e) b2_gamma | b2_delta, and C_h.
   float c1[kMaxHeads][128];
   float b2[kMaxHeads][128];
@@ -95,9 +98,9 @@ struct TcSmem {
   int first_item;  // the first batch's start
 };
 
-// Entry u (0 .. 127) of the vectors of the surrogate head h in slot: of c1, the first layer's context
+// Component u (0 .. 127) of the vectors of the surrogate head h, into an entry: of c1, the first layer's context
 // half folded (a 64-term dot product per hidden unit), and of the second layer's biases and C_h.
-__device__ __noinline__ void head_c1(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int u) {
+__device__ __noinline__ void head_c1(const HeadAttnArgs& a, TcSmem& sm, int entry, int h, int u) {
   const int uu = u & 63;
   const float4* ctx = reinterpret_cast<const float4*>(a.ctx + h * 64);
   const __nv_bfloat16* w = (u < 64 ? a.sw.g1_w : a.sw.d1_w) + ((size_t)h * 64 + uu) * 128 + 64;
@@ -111,12 +114,12 @@ __device__ __noinline__ void head_c1(const HeadAttnArgs& a, TcSmem& sm, int slot
     acc = fmaf(bf16_lo(wv.z), c1.x, fmaf(bf16_hi(wv.z), c1.y, acc));
     acc = fmaf(bf16_lo(wv.w), c1.z, fmaf(bf16_hi(wv.w), c1.w, acc));
   }
-  sm.c1[slot][u] = acc;
+  sm.c1[entry][u] = acc;
 }
-__device__ __forceinline__ void head_out(const HeadAttnArgs& a, TcSmem& sm, int slot, int h, int u) {
+__device__ __forceinline__ void head_out(const HeadAttnArgs& a, TcSmem& sm, int entry, int h, int u) {
   const float b = (u < 64 ? a.sw.g2_b : a.sw.d2_b)[h * 64 + (u & 63)];
-  sm.b2[slot][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
-  if (u < 64) sm.cx[slot][u] = a.ctx[h * 64 + u];
+  sm.b2[entry][u] = u < 64 ? -1.4426950408889634f * b : b;  // gamma's enters sigma's exponent
+  if (u < 64) sm.cx[entry][u] = a.ctx[h * 64 + u];
 }
 
 struct TcMaps {
@@ -463,28 +466,28 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
     bool ok = true;
     // The heads' vectors: all of them now, while the first tile's copies and MMAs run, or with
     // single items (few of a CTA's heads are ever used) each when a tile first needs it.
-    uint32_t ready = 0;  // heads (by slot) whose vectors this warp can read
-    // A head's vectors by the group's warps: an entry of c1 in lanes 0-15, of the rest in 16-31,
+    const bool all_vec = batch > 1;
+    int vec_slot = -1;  // with single items: the head (by slot) whose vectors this warp can read
+    // A head's vectors by the group's warps: a component of c1 in lanes 0-15, of the rest in 16-31,
     // handed over through an mbarrier (a bounded wait, unlike a named barrier).
     uint32_t n_vec = 0;
     auto group_vectors = [&](int slot, int h) -> bool {
       const int u = (4 * part + quarter) * 16 + (lane & 15);
       if (lane < 16)
-        head_c1(a, sm, slot, h, u);
+        head_c1(a, sm, vec_entry(g, n_vec), h, u);
       else
-        head_out(a, sm, slot, h, u);
-      ready |= 1u << slot;
+        head_out(a, sm, vec_entry(g, n_vec), h, u);
+      vec_slot = slot;
       __syncwarp();
       if (elect_one()) mbar_arrive(&sm.vec_full[g]);
       __syncwarp();
       return mbar_wait_warp(&sm.vec_full[g], n_vec++ & 1, err, abort_flag);
     };
-    if (batch > 1) {
+    if (all_vec) {
       for (int i = tid - 64; i < n_surr * 128; i += kGroupThreads * kTcGroups) {
         head_c1(a, sm, i >> 7, a.head_ids[s_first + (i >> 7)], i & 127);
         head_out(a, sm, i >> 7, a.head_ids[s_first + (i >> 7)], i & 127);
       }
-      ready = 0xffffffffu;
       asm volatile("bar.sync 3, %0;" ::"n"(kGroupThreads * kTcGroups) : "memory");
     } else if (g == 0 && first_item < surr_items) {
       ok = group_vectors(first_item / T, a.head_ids[s_first + first_item / T]);
@@ -499,10 +502,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) cheap_heads_tc_kernel(const __g
       const bool surr = it < surr_items;
       const int tile = *reinterpret_cast<volatile int*>(&sm.acc_tile[g]);  // a mean item spans kMeanRows rows
       const int slot = *reinterpret_cast<volatile int*>(&sm.acc_slot[g]);  // surrogate head slot: its vectors
-      if (surr && !((ready >> slot) & 1u) && !group_vectors(slot, h)) break;
-      const float* c1 = sm.c1[slot];
-      const float* b2 = sm.b2[slot];
-      const float* cx = sm.cx[slot];
+      if (surr && !all_vec && slot != vec_slot && !group_vectors(slot, h)) break;
+      const int entry = all_vec ? slot : vec_entry(g, n_vec - 1);
+      const float* c1 = sm.c1[entry];
+      const float* b2 = sm.b2[entry];
+      const float* cx = sm.cx[entry];
       const uint32_t t_d1 = t_grp, t_d2 = t_grp + 128;
       if (surr) {
         // H = 2 GELU(D1 + c1) as bf16 pairs (the factor 2 is exact in bf16 and is taken out
