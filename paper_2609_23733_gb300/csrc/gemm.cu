@@ -27,6 +27,7 @@
 #include <math.h>
 
 #include "common.cuh"
+#include "gemm_drain.h"
 #include "internal.h"
 
 namespace vp {
@@ -59,6 +60,10 @@ struct GemmSmem {
   uint32_t tmem_base;
   uint32_t skip_mask;  // K-blocks left out (LinearArgs::skip_ids)
   int abort_flag;
+  uint32_t peer_abort;   // the other CTA's abort_flag, seen behind the cluster barrier at the end
+  uint32_t res_asked[16], res_done[16];  // per epilogue warp: residual blocks asked for, stored
+  uint32_t issued;       // K blocks whose copies this CTA's producer has issued
+  uint32_t peer_issued;  // leader's: the other CTA's
 };
 static_assert(sizeof(GemmSmem<256>) <= 232448 && sizeof(GemmSmem<128>) <= 232448, "shared memory");
 
@@ -107,6 +112,52 @@ __device__ __forceinline__ TileUnit tile_unit(int u, int full_units, int n_tiles
 
 __device__ unsigned int g_linear_err;  // error word of calls without a workspace (vp_linear)
 
+// After a failed wait in either CTA of a pair, called by all their threads: waits (bounded) until the
+// operand copies that either producer has issued have landed, and the residual blocks asked for, and the
+// MMAs issued have completed.
+template <int kBN, bool kSkip, int kEpiWarps>
+__device__ __noinline__ void drain_pair(int N, int K, int full_units) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  GemmSmem<kBN>& sm = *reinterpret_cast<GemmSmem<kBN>*>(smem_raw);
+  constexpr uint32_t kStages = GemmSmem<kBN>::kStages;
+  const int rank = (int)cluster_cta_rank(), pair = (int)(blockIdx.x >> 1), pairs = (int)(gridDim.x >> 1);
+  const int n_tiles = (N + kBN - 1) / kBN, k_blocks = (K + kBK - 1) / kBK;
+  if (threadIdx.x == 0 && rank == 1) st_cluster_u32(cluster_addr(&sm.peer_issued, 0), sm.issued);
+  cluster_sync_all();
+  if (rank == 0 && threadIdx.x == 0) {
+#pragma unroll 1
+    for (uint32_t s = 0; s < kStages; ++s) {
+      const StageDrain d = stage_drain(sm.issued, sm.peer_issued, s, kStages);
+      if (d.uses == 0) continue;
+      const int unit_blocks = k_blocks - (kSkip ? __popc(sm.skip_mask) : 0);
+      const TileUnit t = tile_unit<kBN>(pair + pairs * (int)(d.block / unit_blocks), full_units, n_tiles);
+      const uint32_t half = kABytes + t.w / 2 * kBK * 2;
+      if (d.fix > 0) mbar_arrive_expect_tx(&sm.full[s], half);
+      if (d.fix < 0) mbar_complete_tx(&sm.full[s], half);
+      for (int it = 0; it < 1000000 && !mbar_try_wait(&sm.full[s], (d.uses - 1) & 1); ++it) {}
+    }
+  }
+  const int warp = warp_uniform_id();
+  if (warp >= 2 && elect_one()) {
+    constexpr uint32_t kBufs = GemmSmem<kBN>::kBlocks / kEpiWarps;
+#pragma unroll 1
+    for (uint32_t n = sm.res_done[warp - 2]; n < sm.res_asked[warp - 2]; ++n) {
+      uint64_t* bar = &sm.res_full[(warp - 2) * kBufs + n % kBufs];
+      for (int it = 0; it < 1000000 && !mbar_try_wait(bar, (n / kBufs) & 1); ++it) {}
+    }
+  }
+  __syncwarp();
+  if (rank == 0 && warp == 1) {
+    if (elect_one()) {  // the lane that issued the MMAs
+      tc_commit_pair(&sm.drain);
+      for (int it = 0; it < 1000000 && !mbar_try_wait(&sm.drain, 0); ++it) {}
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+  cluster_sync_all();
+}
+
 // kSkip: the instance that leaves K-blocks out (GemmParams::skip_ids); the other instance has
 // none of that bookkeeping.
 template <bool kSkip, int kEpiWarps, bool kQk = false, int kBN = 256>
@@ -144,6 +195,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
     for (int b = 0; b < kBlocks; ++b) mbar_init(&sm.res_full[b], 1);
     mbar_init(&sm.drain, 1);
     sm.abort_flag = 0;
+    sm.peer_abort = 0;
     fence_mbarrier_init();
     fence_proxy_async_smem();
     tma_prefetch_desc(&tmap_a);
@@ -214,14 +266,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         ++lc;
       }
     }
-    if (!ok && lane == 0 && rank == 0) {  // both CTAs' copies, as far as they were issued
-      for (int s = 0; s < kStages; ++s) {
-        if (lc > (uint32_t)s) {
-          const uint32_t last = (lc - 1 - s) / kStages * kStages + s;
-          for (int i = 0; i < 1000000 && !mbar_try_wait(&sm.full[s], (last / kStages) & 1); ++i) {}
-        }
-      }
-    }
+    if (lane == 0) sm.issued = lc;
   } else if (warp == 1) {
     // MMA issuer (leader): converged warp; the elected lane (always the lowest, so the same one)
     // issues the MMAs and the commits that track them, which arrive in both CTAs.
@@ -256,13 +301,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       }
       if (!ok) break;
       if (elect_one()) tc_commit_pair(&sm.acc_full[ab]);
-      __syncwarp();
-    }
-    if (!ok) {
-      if (elect_one()) {
-        tc_commit_pair(&sm.drain);
-        for (int it = 0; it < 1000000 && !mbar_try_wait(&sm.drain, 0); ++it) {}
-      }
       __syncwarp();
     }
   } else {
@@ -303,7 +341,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       epi_sync();
       tc_fence_after();
     }
-    uint32_t i = 0, nst = 0;
+    if (elect_one()) sm.res_asked[e] = 0;
+    uint32_t i = 0, nst = 0;  // units, blocks stored
     for (int u = pair; u < prm.units; u += pairs, ++i) {
       const TileUnit t = tile_unit<kBN>(u, prm.full_units, n_tiles);
       const uint32_t ab = i & 1;
@@ -319,7 +358,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
       const bool row_ok = row < M;
       // The tile's residual blocks into the staging blocks (once the stores before have read
       // them) while the tile's MMAs run.
-      if (prm.residual) {
+      if (prm.residual && alive) {
         if (elect_one()) {
           tma_store_wait_read<0>();
           for (int gi = 0; gi < n_grp; ++gi) {
@@ -327,6 +366,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
               const int buf = (nst + gi) % kBufs;
               mbar_arrive_expect_tx(&res_bar[buf], kBlkBytes);
               tma_load_2d(stg + buf * kBlkBytes, &tmap_res, &res_bar[buf], pcol0 + 64 * gi, row0);
+              sm.res_asked[(threadIdx.x >> 5) - 2] = nst + gi + 1;
             }
           }
         }
@@ -644,13 +684,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(64 + 32 * kEpiWarps,
         }
       }
     }
-    if (elect_one()) tma_store_wait_read<0>();  // the staging blocks outlive the reads
+    if (elect_one()) {
+      sm.res_done[(threadIdx.x >> 5) - 2] = nst;
+      tma_store_wait_read<0>();  // the staging blocks outlive the reads
+    }
     __syncwarp();
   }
 
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && sm.abort_flag) st_cluster_u32(cluster_addr(&sm.peer_abort, cluster_cta_rank() ^ 1), 1u);
   cluster_sync_all();  // neither CTA leaves while the other uses its shared memory or TMEM
+  if (sm.abort_flag || sm.peer_abort) drain_pair<kBN, kSkip, kEpiWarps>(prm.N, prm.K, prm.full_units);
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, kTmemCols);
