@@ -301,7 +301,8 @@ void prof_extra_launch();  // one more kernel inside the current bracket
 
 // Launch with programmatic stream serialization: the kernel may start before the one before it
 // in the stream has completed and calls pdl_wait (common.cuh) before it touches what that one
-// reads or writes.
+// reads or writes.  A refused launch is reported by the return value alone: the runtime's last error is
+// cleared, as the caller's next check is not about it.
 template <typename... K, typename... A>
 cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, int threads, size_t smem, cudaStream_t st,
                        A&&... args) {
@@ -315,7 +316,9 @@ cudaError_t launch_pdl(void (*kernel)(K...), dim3 grid, int threads, size_t smem
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
 }
 
 int device_sm_count();
