@@ -174,8 +174,19 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // once the kernel before has completed and its writes are visible; as every kernel waits (all
 // of it, or at least one thread before the grid ends), everything earlier in the stream has
 // completed too.  What an earlier kernel wrote is read with plain loads, never __ldg: the compiler
-// may move a read-only load above the wait.  pdl_launch, after the wait, lets the next kernel start: what that one does
-// before its own wait can rely on every kernel before this one.
+// may move a read-only load above the wait.  pdl_launch lets the next kernel start once every CTA has called
+// it or ended.  Where it comes after the wait, what the next kernel does before its own wait can rely on
+// every kernel before this one.  Kernels that call it before their wait (or do not wait until their end),
+// behind which the kernel before them may still be running too:
+//   attn_full_kernel<true> behind the whole groups.  Its successor (cheap_heads_tc_kernel or
+//     broadcast_heads_kernel) reads bins, C_h, mean of V, QKV and weights and writes its own heads' rows of Y and
+//     W_O's bias ahead of its wait: all of that is settled before the whole-group kernel triggers, which
+//     waits first, and the two attention kernels touch other rows of Y;
+//   cheap_heads_tc_kernel, broadcast_heads_kernel, and ln_fold_kernel with weights_ready.  Their successors (W_O's or
+//     QKV's GEMM, the RoPE table, the first kernel of the next call) touch nothing in global memory ahead of
+//     their wait: no w_ready, no weights_ready behind these.
+// Kernels that read or write global memory ahead of their wait, all behind one that triggers after its own:
+// attn_full_kernel<true> behind the whole groups, ln_fold_kernel with weights_ready, gemm_kernel with w_ready (W alone).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

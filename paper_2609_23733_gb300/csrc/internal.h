@@ -197,8 +197,9 @@ struct LinearArgs {
   // 32 x 64; no LayerNorm fold, no qk columns).  NULL: none.
   const int32_t* skip_ids;
   const int32_t* skip_off;
-  // The kernel just before this one in the stream is the library's own and does not write W: its
-  // first tiles may be read before that kernel has completed.
+  // The kernel just before this one in the stream is the library's own, triggers after its own wait
+  // (pdl_launch, common.cuh) and does not write W: W's first tiles may be read before that kernel has
+  // completed.
   bool w_ready;
 };
 cudaError_t launch_linear(const LinearArgs& a, int num_sms, cudaStream_t st);
@@ -216,8 +217,9 @@ cudaError_t launch_wo_mean_fold(int D, int H, const __nv_bfloat16* w_o, const fl
 cudaError_t launch_ln_partials(int M, int D, const __nv_bfloat16* x, float2* part, cudaStream_t st);
 // The folded LayerNorm's weights for a projection W [Nout][K] (nn.Linear layout):
 // Wp = W diag(g) (bf16), c[o] = sum_k Wp[o][k] (of the bf16 Wp), bp[o] = b[o] + sum_k W[o][k] beta[k]
-// (b NULL: 0).  K % 256 == 0, K <= 4096.  weights_ready: no kernel just before writes W, g, beta or b,
-// and none reads the outputs any more (see ln_fold_kernel).
+// (b NULL: 0).  K % 256 == 0, K <= 4096.  weights_ready: the kernel just before is the
+// library's own, triggers after its own wait, does not write W, g, beta or b and does not read the outputs
+// (see ln_fold_kernel).
 // cos / sin of p * base^(-i / 16), p = 0 .. max_pos, i = 0 .. 15: table [i / 2][max_pos + 1][i % 2].
 cudaError_t launch_rope_table(int max_pos, float base, float2* table, cudaStream_t st);
 cudaError_t launch_ln_fold_weights(int Nout, int K, const __nv_bfloat16* W, const float* g,

@@ -157,9 +157,9 @@ __global__ void __launch_bounds__(256) ln_partials_kernel(int M, const __nv_bflo
 
 // Folded LayerNorm weights: one warp per output row o of W [Nout][K]; lane l holds the
 // 16-byte chunks c 32 + l of the row.  With weights_ready W is a weight (not another kernel's
-// output) and the outputs' last readers have completed when the kernel may start (every kernel
-// lets the next one start after its own wait): it then runs beside the kernel before it (the
-// previous block's FFN-down) and waits only at its end.
+// output) and the outputs' last readers have completed when the kernel may start, because the kernel
+// before it (the previous block's FFN-down, or the input's statistics pass) triggers after its own
+// wait: it then runs beside that one and waits only at its end.
 template <int C>
 __global__ void __launch_bounds__(256) ln_fold_kernel(int Nout, const __nv_bfloat16* W,
                                                       const float* g, const float* beta,
