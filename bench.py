@@ -848,17 +848,27 @@ def kernel_case(args):
     print(json.dumps({"kernel_case": args.kernel_case, "tokens": N, "launches": args.case_launches}))
 
 
+# Files that a kernel's traffic follows from: its code, its plan of the work and the layout of its scratch.
+TRAFFIC_SOURCES = {"attn_full": ("attn_full.cu", "attn_plan.cuh", "attn_split.h"), "gemm": ("gemm.cu", "gemm_drain.h")}
+
+
+def source_hash(kernel):
+    h = hashlib.sha256()
+    for name in TRAFFIC_SOURCES[kernel]:
+        with open(os.path.join(ROOT, "paper_2609_23733_gb300", "csrc", name), "rb") as f:
+            h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def traffic_from_profile(kernel):
-    """DRAM bytes per launch from the committed ncu summary, if the kernel source still
-    matches the hash recorded there (else None)."""
+    """DRAM bytes per launch from the committed ncu summary, if the kernel's sources still
+    match the hash recorded there (else None)."""
     path = os.path.join(ROOT, "profiles", f"{kernel}_traffic.txt")
-    src = {"attn_full": "attn_full.cu", "gemm": "gemm.cu"}[kernel]
     try:
         kv = dict(line.strip().split("=", 1) for line in open(path) if "=" in line and not line.startswith("#"))
     except OSError:
         return None
-    h = hashlib.sha256(open(os.path.join(ROOT, "paper_2609_23733_gb300", "csrc", src), "rb").read()).hexdigest()[:16]
-    if kv.get("source_sha256_16") != h:
+    if kv.get("source_sha256_16") != source_hash(kernel):
         return None
     try:
         return float(kv["dram_bytes_per_launch_scaled"])
