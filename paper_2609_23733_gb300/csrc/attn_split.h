@@ -32,11 +32,12 @@ constexpr int kMaxTailUnits = kFaTailUnits * 4 / kFaChains;
 // 2,748 to 137,400 tokens; being costs in time they do not shrink with n_kv.  (13 and 1.5, which fitted
 // while a group's last part combined it, took 1.1 % longer in the mean of 17 shapes: 3 heads at
 // 10,992 tokens 116.7 us against 111.8, 1 at 15,432 84.0 against 79.7, at 43,968 435 against 432.)
-// Against a share of 3 % of a group per part, which took as many parts as CTAs: 16 heads at
-// 10,992 tokens 466 -> 383 us (8 groups left over: 19 parts -> 13), 3 heads 166 -> 112, 1 head at
-// 15,432 tokens 101 -> 80.  Below kShortTiles the choice of S is worth less than 5 us (1,044 tokens:
-// 28 us for every S up to 10, 32 for the 17 that the share rule takes), and the share rule stays
-// there: a deep stack of short sequences then gives the same bits as it always did.
+// Against a share of 3 % of a group per part at every length (captured calls with 6 surrogate heads beside):
+// 16 heads at 10,992 tokens 390 -> 384 us (8 groups left over, 19 parts -> 13), one head at 43,968 478 -> 463
+// (115 groups, whole -> 5 parts), at 137,400 3,785 -> 3,670 (54 groups, 5 -> 11); the same within 1 % for 3
+// heads at 10,992 and one at 15,432.  Below kShortTiles the share rule stays although fewer parts are quicker
+// (1,044 tokens: 4 heads 25.2 us with its 12 parts, 18.5 with 6 to 8; one head 18.5 with 17, 17.2 with 8): a
+// deep stack of short sequences, which amplifies any other rounding, then gives the bits it always gave.
 constexpr int kMaxParts = 64;
 constexpr int kUnitTiles = 7, kCombineTiles = 1;
 constexpr int kShortTiles = 41;

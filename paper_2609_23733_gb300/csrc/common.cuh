@@ -185,8 +185,9 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 //   cheap_heads_tc_kernel, broadcast_heads_kernel, and ln_fold_kernel with weights_ready.  Their successors (W_O's or
 //     QKV's GEMM, the RoPE table, the first kernel of the next call) touch nothing in global memory ahead of
 //     their wait: no w_ready, no weights_ready behind these.
-// Kernels that read or write global memory ahead of their wait, all behind one that triggers after its own:
-// attn_full_kernel<true> behind the whole groups, ln_fold_kernel with weights_ready, gemm_kernel with w_ready (W alone).
+// Beside those two successors, three read or write global memory ahead of their wait, each behind a kernel that
+// triggers after its own: attn_full_kernel<true> behind the whole groups, ln_fold_kernel with weights_ready,
+// gemm_kernel with w_ready (W alone).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
