@@ -31,11 +31,13 @@ __device__ __forceinline__ Plan make_plan(int G, int P, int n_kv, bool parts_onl
   pl.S = 1;
   if (pl.T > 0) {
     const int s0 = lane_id() + 1, s1 = s0 + 32;
-    const uint32_t c0 = split_allowed(pl.T, n_kv, s0) ? split_cost(pl.T, P, n_kv, s0) : 0xffffffffu;
-    const uint32_t c1 = split_allowed(pl.T, n_kv, s1) ? split_cost(pl.T, P, n_kv, s1) : 0xffffffffu;
-    const uint32_t best = __reduce_min_sync(0xffffffffu, min(c0, c1));
-    const uint32_t lo = __ballot_sync(0xffffffffu, c0 == best), hi = __ballot_sync(0xffffffffu, c1 == best);
-    pl.S = lo ? __ffs(lo) : 32 + __ffs(hi);
+    auto cheapest = [](uint32_t c0, uint32_t c1) -> int {
+      const uint32_t best = __reduce_min_sync(0xffffffffu, min(c0, c1));
+      const uint32_t lo = __ballot_sync(0xffffffffu, c0 == best), hi = __ballot_sync(0xffffffffu, c1 == best);
+      return lo ? __ffs(lo) : 32 + __ffs(hi);
+    };
+    pl.S = cheapest(share_cost(pl.T, P, n_kv, s0), share_cost(pl.T, P, n_kv, s1));
+    pl.S = cheapest(split_cost(pl.T, P, n_kv, s0, pl.S), split_cost(pl.T, P, n_kv, s1, pl.S));
   }
   pl.units = pl.S == 1 ? G : pl.R * P + pl.T * pl.S;
   pl.whole = parts_only ? 0 : (pl.S == 1 ? G : pl.R * P);
